@@ -419,7 +419,7 @@ apip_status energy_forces_t(apip_ctx* c, const double* pos, const int32_t* id, i
   if (e_total) {
     Phase ph(c, APIP_PHASE_REDUCE, 1, s);
     launch_final(c->partials, a.n_part_p1 + c->ace_blocks, e_total, nullptr, nullptr, 0, nullptr,
-                 c->flags, c->counts, nullptr, c->cell_count, c->ncell, s);
+                 c->flags, c->counts, nullptr, c->cell_count, c->ncell, c->e_scratch, c->counts + 2, s);
   }
   if (a.ind_on) launch_ind_work(c->ind_acc, 0.0, a.det, s);
   return launch_status(c);
@@ -440,7 +440,7 @@ apip_status switch_t(apip_ctx* c, const double* pos, const int32_t* id, int n, d
   if (lam_out) launch_get_field<T>(a, APIP_FIELD_LAM, lam_out, s);
   if (dlam_out) launch_get_field<T>(a, APIP_FIELD_DLAM, dlam_out, s);
   launch_final(c->partials, 0, nullptr, nullptr, nullptr, 0, nullptr, c->flags, c->counts, n_ace_out, c->cell_count,
-               c->ncell, s);
+               c->ncell, c->e_scratch, c->counts + 2, s);
   return launch_status(c);
 }
 
@@ -481,13 +481,14 @@ apip_status verlet_t(apip_ctx* c, double* pos, double* vel, double* force, const
     if (thermo) {
       Phase ph(c, APIP_PHASE_REDUCE, 1, s);
       launch_final(c->partials, n_part, nullptr, thermo + 5 * k, k > 0 ? tp : nullptr, ntb,
-                   k > 0 ? thermo + 5 * (k - 1) : nullptr, c->flags, c->counts, nullptr, c->cell_count, c->ncell, s);
+                   k > 0 ? thermo + 5 * (k - 1) : nullptr, c->flags, c->counts, nullptr, c->cell_count, c->ncell, c->e_scratch, c->counts + 2, s);
     }
   }
   { NvtxRange nv("apip.prep"); Phase ph(c, APIP_PHASE_PREP, 1, s); launch_verlet<T>(a, 2, pos, vel, force, inv_mass, dt, tp, s); }
   if (thermo) {
     Phase ph(c, APIP_PHASE_REDUCE, 1, s);
-    launch_thermo_final(c->thermo_part, ntb, thermo + 5 * (steps - 1), s);
+    launch_final(c->partials, 0, nullptr, nullptr, c->thermo_part, ntb, thermo + 5 * (steps - 1), nullptr, c->counts,
+                 nullptr, nullptr, 0, c->e_scratch, c->counts + 2, s);
   }
   return launch_status(c);
 }
@@ -629,7 +630,7 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
   const int p1 = (int)std::max<int64_t>(nblk(n_atoms_max), (n_atoms_max + kLearnedBlock - 1) / kLearnedBlock);
   APIP_ALLOC(ctx->partials, sizeof(double) * (p1 + ctx->ace_blocks));
   APIP_ALLOC(ctx->thermo_part, sizeof(double) * 4 * p1);
-  APIP_ALLOC(ctx->e_scratch, sizeof(double) * 2);
+  APIP_ALLOC(ctx->e_scratch, sizeof(double) * kFinalScratch);
   APIP_ALLOC(ctx->ind_acc, sizeof(double) * 3);
   APIP_ALLOC(ctx->mlp_w, es * APIP_MLP_NPARAM);
   if (p->precision == APIP_FP32) {

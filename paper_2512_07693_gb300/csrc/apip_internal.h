@@ -17,6 +17,9 @@ constexpr int kLmaxCap = 4;    // largest l_max
 constexpr int kCspCap = 8;     // largest csp_nnb
 constexpr int kBlock = 256;    // threads per block of the all-atom passes
 constexpr int kLearnedBlock = 128;   // threads per block of pass 1 with the learned switch
+constexpr int kFinalThreads = 64;            // threads per block of the step's float64 sums
+constexpr int kFinalBlocks = 128;            // most blocks of them (fewer than two per SM)
+constexpr int kFinalScratch = kFinalBlocks * (kFinalThreads / 32) * 5 * 2;   // doubles: (sum, compensation) per warp and value
 constexpr int kAceWarps = 8;               // warps per ACE block
 constexpr int kAceThreads = 32 * kAceWarps;
 
@@ -179,14 +182,14 @@ struct apip_ctx {
   double* cvec = nullptr;      // [nmax] grad-lambda CSP coefficients (kept zero between calls)
   int* ace_list = nullptr;     // [nmax]
   int* clist = nullptr;        // [nmax] learned switch: atoms with a grad-lambda coefficient
-  int* counts = nullptr;       // [4]: |P|, learned c-vector count, scratch
+  int* counts = nullptr;       // [4]: |P|, learned c-vector count, k_final's ticket (zero between launches)
   int* blk_cnt = nullptr;      // deterministic mode: pass 2's per-block counts of lam > 0, then their offsets
   bool det = false;            // apip_params.deterministic
   int* flags = nullptr;        // [4]: need_rebuild, largest squared displacement since the build (float bits)
   int* status = nullptr;       // [ST_COUNT]
   double* partials = nullptr;  // energy partials: P1 blocks then ACE warps
   double* thermo_part = nullptr;  // [blocks][4] KE, px, py, pz
-  double* e_scratch = nullptr;    // [2] total energy scratch
+  double* e_scratch = nullptr;    // [kFinalScratch] per-warp sums of k_final
   int n_part = 0;
   int ace_blocks = 0;
 

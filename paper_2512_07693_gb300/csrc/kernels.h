@@ -126,8 +126,10 @@ __device__ __forceinline__ int bounds_check(int* status, int site, int v, int li
 __device__ __forceinline__ void end_list_build(int* flags, int* cell_count, int ncell) {
   const int built = flags[0];
   __syncthreads();
-  if (built)
-    for (int c = threadIdx.x; c < ncell; c += blockDim.x) cell_count[c] = 0;
+  if (built) {   // 16-byte stores (the counters start on an allocation boundary), then the last few
+    for (int c = threadIdx.x; c < ncell / 4; c += blockDim.x) reinterpret_cast<int4*>(cell_count)[c] = make_int4(0, 0, 0, 0);
+    if (threadIdx.x < (ncell & 3)) cell_count[(ncell & ~3) + threadIdx.x] = 0;
+  }
   if (threadIdx.x == 0) flags[0] = 0;
 }
 
@@ -243,9 +245,13 @@ template <typename T> void launch_fm_buffer(const Args<T>& a, cudaStream_t s);
 void launch_ind_work(double* acc, double dt, int det, cudaStream_t s);
 void launch_fix_finish(double* force, int n, cudaStream_t s);
 template <typename T> void launch_csp_force(const Args<T>& a, cudaStream_t s);
+// the step's float64 sums (n_part energy partials, n_tblocks x 4 thermo partials, each
+// optional); scratch holds kFinalScratch doubles, *ticket is zero between launches;
+// flags (optional): the list-build trigger to clear
 void launch_final(double* partials, int n_part, double* e_total, double* e_pot_slot,
                   const double* thermo_part, int n_tblocks, double* thermo_slot, int* flags,
-                  const int* counts, int64_t* n_ace_out, int* cell_count, int ncell, cudaStream_t s);
+                  const int* counts, int64_t* n_ace_out, int* cell_count, int ncell, double* scratch, int* ticket,
+                  cudaStream_t s);
 template <typename T> void launch_get_field(const Args<T>& a, int field, void* dst, cudaStream_t s);
 void launch_fill_const_list(int* list, int* counts, int n, cudaStream_t s);
 
@@ -254,7 +260,6 @@ void launch_fill_const_list(int* list, int* counts, int n, cudaStream_t s);
 template <typename T> void launch_verlet(const Args<T>& a, int mode, double* pos, double* vel,
                                          const double* force, const double* inv_mass, double dt,
                                          double* thermo_part, cudaStream_t s);
-void launch_thermo_final(const double* thermo_part, int n_tblocks, double* thermo_slot, cudaStream_t s);
 
 // learned indicator (kernels_mlp.cu)
 template <typename T> void launch_pass1_learned(const Args<T>& a, cudaStream_t s);

@@ -5,6 +5,8 @@
 // float64 reductions and the velocity-Verlet kernels.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "kernels.h"
 
 namespace apip {
@@ -753,38 +755,77 @@ __device__ __forceinline__ void neumaier(double& s, double& c, double v) {
   s = t;
 }
 
-__global__ void k_final(const double* partials, int n_part, double* e_total, double* e_pot_slot,
-                        const double* thermo_part, int n_tb, double* thermo_slot, int* flags,
-                        const int* counts, int64_t* n_ace_out, int* cell_count, int ncell) {
+// The float64 sums of a step, in one launch of many small blocks: the energy
+// partials (value 0) and, with thermo, the four kinetic-energy and momentum
+// partials per block of the Verlet kernel (values 1..4).
+//
+// What bounds it: an SM does two float64 additions a cycle, so one block that sums
+// everything (972 x 5 partials for 249 k atoms, 15 600 x 5 for 4 M) takes its time in
+// its own float64 pipe: 23 us at 249 k atoms.  With a partial or two per thread in
+// 64-thread blocks over all SMs (whole step with thermo output, same run: 225.1 ->
+// 217.5 us at 249 k atoms, 2.307 -> 2.163 ms at 4 M) the
+// additions cost nothing; what is left is the latency of two dependent passes.  Each warp leaves its compensated sums (s, c) in
+// scratch[warp][value][2]; the block that draws the last ticket adds them in warp
+// order, so the sum does not depend on the order of the blocks.
+__global__ void __launch_bounds__(kFinalThreads)
+    k_final(const double* partials, int n_part, double* e_total, double* e_pot_slot, const double* thermo_part,
+            int n_tb, double* thermo_slot, int* flags, const int* counts, int64_t* n_ace_out, int* cell_count, int ncell,
+            double* scratch, int* ticket) {
   pdl_begin();
-  end_list_build(flags, cell_count, ncell);
-  __shared__ double sh[32];
-  double s = 0.0, c = 0.0;
-  for (int k = threadIdx.x; k < n_part; k += blockDim.x) neumaier(s, c, partials[k]);
-  const double tot = block_sum(s, sh) + block_sum(c, sh);
-  if (threadIdx.x == 0) {
-    if (e_total) *e_total = tot;
-    if (e_pot_slot) *e_pot_slot = tot;
-    if (n_ace_out) *n_ace_out = (int64_t)counts[0];
-  }
-  if (thermo_part) {
-    for (int q = 0; q < 4; ++q) {
-      double ts = 0.0, tc = 0.0;
-      for (int k = threadIdx.x; k < n_tb; k += blockDim.x) neumaier(ts, tc, thermo_part[4 * k + q]);
-      const double tt = block_sum(ts, sh) + block_sum(tc, sh);
-      if (threadIdx.x == 0) thermo_slot[1 + q] = q == 0 ? 0.5 * tt : tt;   // partials hold 2 E_kin
+  if (flags && blockIdx.x == 0) end_list_build(flags, cell_count, ncell);
+  constexpr int kWarps = kFinalThreads / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int t0 = blockIdx.x * kFinalThreads + threadIdx.x, stride = gridDim.x * kFinalThreads;
+  double s[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, c[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+  for (int k = t0; k < n_part; k += stride) neumaier(s[0], c[0], partials[k]);
+  if (thermo_part)
+    for (int k = t0; k < n_tb; k += stride) {
+      const double2 u = reinterpret_cast<const double2*>(thermo_part)[2 * k];
+      const double2 v = reinterpret_cast<const double2*>(thermo_part)[2 * k + 1];
+      neumaier(s[1], c[1], u.x);
+      neumaier(s[2], c[2], u.y);
+      neumaier(s[3], c[3], v.x);
+      neumaier(s[4], c[4], v.y);
+    }
+  const int nq = thermo_part ? 5 : 1;
+  for (int q = 0; q < nq; ++q) {
+    const double ts = warp_sum(s[q]);
+    const double tc = warp_sum(c[q]);
+    if (lane == 0) {
+      double* out = scratch + ((size_t)(blockIdx.x * kWarps + warp) * 5 + q) * 2;
+      out[0] = ts;
+      out[1] = tc;
     }
   }
-}
-
-__global__ void k_thermo_final(const double* thermo_part, int n_tb, double* thermo_slot) {
-  pdl_begin();
-  __shared__ double sh[32];
-  for (int q = 0; q < 4; ++q) {
+  __shared__ int last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const int nw = gridDim.x * kWarps;
+  for (int q = warp; q < nq; q += kWarps) {
     double ts = 0.0, tc = 0.0;
-    for (int k = threadIdx.x; k < n_tb; k += blockDim.x) neumaier(ts, tc, thermo_part[4 * k + q]);
-    const double tt = block_sum(ts, sh) + block_sum(tc, sh);
-    if (threadIdx.x == 0) thermo_slot[1 + q] = q == 0 ? 0.5 * tt : tt;   // partials hold 2 E_kin
+    for (int w = lane; w < nw; w += 32) {
+      const double* in = scratch + ((size_t)w * 5 + q) * 2;
+      neumaier(ts, tc, __ldcg(in));
+      tc += __ldcg(in + 1);
+    }
+    const double tot = warp_sum(ts) + warp_sum(tc);
+    if (lane != 0) continue;
+    if (q == 0) {
+      if (e_total) *e_total = tot;
+      if (e_pot_slot) *e_pot_slot = tot;
+    } else {
+      thermo_slot[q] = q == 1 ? 0.5 * tot : tot;   // partials hold 2 E_kin
+    }
+  }
+  if (threadIdx.x == 0) {
+    if (n_ace_out) *n_ace_out = (int64_t)counts[0];
+    *ticket = 0;
   }
 }
 
@@ -965,13 +1006,12 @@ template <typename T> void launch_csp_force(const Args<T>& a, cudaStream_t s) {
 
 void launch_final(double* partials, int n_part, double* e_total, double* e_pot_slot,
                   const double* thermo_part, int n_tblocks, double* thermo_slot, int* flags,
-                  const int* counts, int64_t* n_ace_out, int* cell_count, int ncell, cudaStream_t s) {
-  launch_pdl(k_final, 1, 256, 0, s, partials, n_part, e_total, e_pot_slot, thermo_part, n_tblocks, thermo_slot,
-                            flags, counts, n_ace_out, cell_count, ncell);
-}
-
-void launch_thermo_final(const double* thermo_part, int n_tblocks, double* thermo_slot, cudaStream_t s) {
-  launch_pdl(k_thermo_final, 1, 256, 0, s, thermo_part, n_tblocks, thermo_slot);
+                  const int* counts, int64_t* n_ace_out, int* cell_count, int ncell, double* scratch, int* ticket,
+                  cudaStream_t s) {
+  const int most = n_part > n_tblocks ? n_part : n_tblocks;
+  const int grid = std::min(nblocks(most, kFinalThreads), kFinalBlocks);
+  launch_pdl(k_final, grid, kFinalThreads, 0, s, partials, n_part, e_total, e_pot_slot, thermo_part, n_tblocks,
+             thermo_slot, flags, counts, n_ace_out, cell_count, ncell, scratch, ticket);
 }
 
 template <typename T> void launch_verlet(const Args<T>& a, int mode, double* pos, double* vel,
