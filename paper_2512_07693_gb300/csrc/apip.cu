@@ -91,10 +91,10 @@ void free_all(apip_ctx* c) {
   for (cudaEvent_t e : c->prof_pool) cudaEventDestroy(e);
   c->prof_pending.clear();
   c->prof_pool.clear();
-  void* ptrs[] = {c->cell_count, c->cell_atoms, c->cell_q, c->nnb, c->nnb_e, c->nnb_0, c->mind1, c->posg, c->nbl, c->nbl_tmp, c->pos_ref, c->posq, c->posq_ref, c->id2idx,
+  void* ptrs[] = {c->cell_count, c->cell_q, c->nnb, c->nnb_e, c->nnb_0, c->mind1, c->posg, c->nbl, c->nbl_tmp, c->pos_ref, c->posq, c->posq_ref, c->id2idx,
                   c->csp, c->csp_idx, c->csp_owner, c->zeta, c->xi_p, c->e_eam, c->g, c->wbar, c->dd, c->lam, c->dlam, c->e_ace,
                   c->cvec, c->ace_list, c->clist, c->counts, c->flags, c->status, c->partials, c->thermo_part,
-                  c->e_scratch, c->ind_acc, c->blk_cnt, c->ace_tab, c->mlp_w, c->mlp_img, c->mlp_x0, c->mlp_ws};
+                  c->e_scratch, c->ind_acc, c->blk_cnt, c->ace_tab, c->mlp_w, c->mlp_img, c->mlp_x0, c->mlp_ws, c->pair_keep};
   for (void* q : ptrs)
     if (q) cudaFree(q);
 }
@@ -148,6 +148,7 @@ apip_status set_geometry(apip_ctx* ctx, const double* box, cudaStream_t s) {
     if (g.nc[k] < 3)
       return fail(ctx, APIP_ERR_ARG, "each box edge must be >= 3 * (cutoff + skin) = " + std::to_string(3 * ctx->r_list));
     g.cs[k] = box[k] / g.nc[k];
+    g.csf[k] = (float)g.cs[k];
     g.invL[k] = 1.0 / box[k];
     g.inv_unit[k] = 4294967296.0 / box[k];
     int x = 0;
@@ -159,19 +160,12 @@ apip_status set_geometry(apip_ctx* ctx, const double* box, cudaStream_t s) {
   }
   if (ncell > ctx->ncell_alloc) {
     if (ctx->cell_count) cudaFree(ctx->cell_count);
-    if (ctx->cell_atoms) cudaFree(ctx->cell_atoms);
     if (ctx->cell_q) cudaFree(ctx->cell_q);
     ctx->cell_count = nullptr;
-    ctx->cell_atoms = nullptr;
     ctx->cell_q = nullptr;
     APIP_CK(cudaMalloc(&ctx->cell_count, sizeof(int) * ncell));
     APIP_CK(cudaMemsetAsync(ctx->cell_count, 0, sizeof(int) * ncell, s));
-    // members: FP64 path their indices, FP32 path their fixed-point positions with
-    // the index in .w
-    if (ctx->p.precision == APIP_FP32)
-      APIP_CK(cudaMalloc(&ctx->cell_q, sizeof(uint4) * (size_t)ncell * ctx->p.cell_cap));
-    else
-      APIP_CK(cudaMalloc(&ctx->cell_atoms, sizeof(int) * (size_t)ncell * ctx->p.cell_cap));
+    APIP_CK(cudaMalloc(&ctx->cell_q, sizeof(uint4) * (size_t)ncell * ctx->p.cell_cap));
     ctx->ncell_alloc = ncell;
   }
   ctx->ncell = ncell;
@@ -262,12 +256,20 @@ Args<T> make_args(apip_ctx* c, const double* pos, const int* id, int n, double* 
   // moved less than skin / 2); the margin covers the rounding of the trigger
   a.r_e_in2 = p.eam_rc * p.eam_rc;
   a.r_e_mid2 = (p.eam_rc + p.skin + 1e-3) * (p.eam_rc + p.skin + 1e-3);
+  a.r_e_in2f = (float)a.r_e_in2;
+  a.r_e_mid2f = (float)a.r_e_mid2;
+  a.r_list2f = (float)a.r_list2;
+  if ((double)a.r_list2f < a.r_list2) a.r_list2f = std::nextafter(a.r_list2f, INFINITY);
+  a.r_scan2f = std::nextafter((float)(a.r_list2 * (1.0 + 4e-5)), INFINITY);
+  a.lanes = atom_lanes(n, c->sms);
+  a.pair_keep = static_cast<double2*>(c->pair_keep);
+  a.pair_rows = p.lam_mode == APIP_LAM_LEARNED ? 0 : c->pair_rows;   // (the learned pass 1 keeps none)
   a.csp_rcut2 = p.csp_rcut * p.csp_rcut;
   a.pos = pos;
   a.id = id;
   a.nnb_e = c->nnb_e; a.nnb_0 = c->nnb_0; a.mind1 = c->mind1; a.posg = c->posg;
   a.nnb = c->nnb; a.nbl = c->nbl; a.nbl_tmp = c->nbl_tmp; a.pos_ref = c->pos_ref; a.posq = c->posq; a.posq_ref = c->posq_ref;
-  a.id2idx = c->id2idx; a.csp = c->csp; a.csp_idx = c->csp_idx; a.csp_owner = c->csp_owner; a.cell_count = c->cell_count; a.cell_atoms = c->cell_atoms;
+  a.id2idx = c->id2idx; a.csp = c->csp; a.csp_idx = c->csp_idx; a.csp_owner = c->csp_owner; a.cell_count = c->cell_count;
   a.ncell = c->ncell;
   a.cell_q = c->cell_q;
   a.zeta = as<T>(c->zeta); a.xi_p = as<T>(c->xi_p); a.e_eam = as<T>(c->e_eam); a.g = as<T>(c->g);
@@ -278,7 +280,7 @@ Args<T> make_args(apip_ctx* c, const double* pos, const int* id, int n, double* 
   a.det = c->det ? 1 : 0; a.blk_cnt = c->blk_cnt;
   a.partials = c->partials;
   // one energy partial per pass-1 block, ahead of the ACE blocks' partials
-  if (p.lam_mode != APIP_LAM_LEARNED) a.n_part_p1 = nblk(n);
+  if (p.lam_mode != APIP_LAM_LEARNED) a.n_part_p1 = nblk((int64_t)n * a.lanes);
   else if (sizeof(T) == 4) a.n_part_p1 = nblk(n);   // the descriptor kernel's blocks
   else a.n_part_p1 = (int)std::max<int64_t>(1, (n + kLearnedBlock - 1) / kLearnedBlock);
   a.force = force;
@@ -300,7 +302,14 @@ namespace {
 template <typename T> void set_view(Args<T>& a, apip_ctx* c);
 template <> void set_view<double>(Args<double>& a, apip_ctx* c) {
   a.pv.pos = a.pos;
-  for (int k = 0; k < 3; ++k) { a.pv.L[k] = c->geo.L[k]; a.pv.invL[k] = 1.0 / c->geo.L[k]; }
+  for (int k = 0; k < 3; ++k) {
+    a.pv.L[k] = c->geo.L[k];
+    a.pv.invL[k] = 1.0 / c->geo.L[k];
+    const double half = 0.5 * c->geo.L[k];
+    unsigned long long bits;
+    std::memcpy(&bits, &half, sizeof(bits));
+    a.pv.half_hi[k] = (int)(bits >> 32);
+  }
 }
 template <> void set_view<float>(Args<float>& a, apip_ctx* c) {
   a.pv.q = c->posq;
@@ -552,6 +561,7 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
   cudaGetDevice(&ctx->dev);
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->dev);
+  ctx->sms = std::max(1, sms);
   // atoms per ACE block.  Pool kernel: the largest group whose pools leave room
   // for two resident blocks per SM, else the largest that fits.  Streamed
   // kernel: 8 atoms per block for the adaptive switches (a few thousand
@@ -601,11 +611,11 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
   const size_t es = esize(ctx);
   APIP_ALLOC(ctx->nnb, sizeof(int) * N);
   APIP_ALLOC(ctx->nnb_e, sizeof(int) * N);
+  APIP_ALLOC(ctx->nnb_0, sizeof(int) * N);
   APIP_ALLOC(ctx->nbl, sizeof(int) * N * p->max_nb);
   APIP_ALLOC(ctx->nbl_tmp, sizeof(int) * N * p->max_nb);
   APIP_ALLOC(ctx->pos_ref, sizeof(double) * 3 * N);
   if (p->precision == APIP_FP32) {
-    APIP_ALLOC(ctx->nnb_0, sizeof(int) * N);
     APIP_ALLOC(ctx->mind1, sizeof(float) * N);
     APIP_ALLOC(ctx->posq, sizeof(uint4) * N);
     APIP_ALLOC(ctx->posq_ref, sizeof(uint4) * N);
@@ -617,6 +627,17 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
   APIP_ALLOC(ctx->csp_owner, sizeof(int) * N);
   void** per_atom[] = {&ctx->zeta, &ctx->xi_p, &ctx->e_eam, &ctx->g, &ctx->wbar, &ctx->dd, &ctx->lam, &ctx->dlam, &ctx->e_ace};
   for (void** q : per_atom) APIP_ALLOC(*q, es * N);
+  if (p->precision == APIP_FP64) {
+    // pass 1's pair terms for pass 2: class 0 of the list (within the EAM cutoff) is
+    // less than half of it.  An entry beyond these rows is computed again, so is
+    // every entry where there is no room for them
+    ctx->pair_rows = (p->max_nb + 1) / 2;
+    if (cudaMalloc(&ctx->pair_keep, sizeof(double2) * N * ctx->pair_rows) != cudaSuccess) {
+      cudaGetLastError();
+      ctx->pair_keep = nullptr;
+      ctx->pair_rows = 0;
+    }
+  }
   APIP_ALLOC(ctx->cvec, sizeof(double) * N);
   APIP_ALLOC(ctx->ace_list, sizeof(int) * N);
   if (p->lam_mode == APIP_LAM_LEARNED) APIP_ALLOC(ctx->clist, sizeof(int) * N);
@@ -626,8 +647,9 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
   APIP_ALLOC(ctx->flags, sizeof(int) * 4);
   APIP_ALLOC(ctx->status, sizeof(int) * ST_COUNT);
   // pass-1 partials: the most blocks either pass 1 launches (the learned one has
-  // smaller blocks)
-  const int p1 = (int)std::max<int64_t>(nblk(n_atoms_max), (n_atoms_max + kLearnedBlock - 1) / kLearnedBlock);
+  // smaller blocks), or a small system's with several threads per atom (atom_lanes)
+  const int p1 = (int)std::max<int64_t>(std::max(nblk(n_atoms_max), 4 * ctx->sms + 1),
+                                        (n_atoms_max + kLearnedBlock - 1) / kLearnedBlock);
   APIP_ALLOC(ctx->partials, sizeof(double) * (p1 + ctx->ace_blocks));
   APIP_ALLOC(ctx->thermo_part, sizeof(double) * 4 * p1);
   APIP_ALLOC(ctx->e_scratch, sizeof(double) * kFinalScratch);
@@ -755,6 +777,7 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
   if (e == cudaSuccess && ctx->posq_ref) e = cudaMemset(ctx->posq_ref, 0, sizeof(uint4) * N);
   if (e == cudaSuccess) e = cudaMemset(ctx->nnb, 0, sizeof(int) * N);
   if (e == cudaSuccess) e = cudaMemset(ctx->nnb_e, 0, sizeof(int) * N);
+  if (e == cudaSuccess) e = cudaMemset(ctx->nnb_0, 0, sizeof(int) * N);
   if (e != cudaSuccess) return fail_create(e);
   double norms[(kLmaxCap + 1) * (kLmaxCap + 1)];
   ylm_norms(kLmaxCap, norms);

@@ -52,6 +52,7 @@ enum {
 struct Geo {
   double L[3];          // box edges
   double cs[3];         // cell edges (>= r_list)
+  float csf[3];         // ... rounded to float
   double invL[3];       // 1 / L
   int nc[3];            // cells per axis (>= 3)
   double inv_unit[3];   // 2^32 / L (FP32 path fixed-point coordinates) = unit_m 2^unit_s,
@@ -142,6 +143,7 @@ struct apip_ctx {
   apip_params p;
   int64_t nmax = 0;
   int dev = 0;
+  int sms = 1;                 // SMs of the device
   double r_list = 0.0;
   apip::Geo geo{};
   bool geo_set = false;
@@ -158,11 +160,10 @@ struct apip_ctx {
 
   // neighbour structures
   int* cell_count = nullptr;   // binning counters, zero outside a list build (read by the fill)
-  uint4* cell_q = nullptr;     // FP32 path: posq of the cell members in cell order
-  int* cell_atoms = nullptr;
+  uint4* cell_q = nullptr;     // cell members' positions (FP32: fixed point; FP64: float, relative to the cell), index
   int* nnb = nullptr;
   int* nnb_e = nullptr;        // entries within eam_rc + skin at build time (they come first)
-  int* nnb_0 = nullptr;        // FP32 path: entries within eam_rc at build time (they come first)
+  int* nnb_0 = nullptr;        // entries within eam_rc at build time (they come first)
   float* mind1 = nullptr;      // FP32 path: least squared build distance of the entries in [eam_rc, eam_rc + skin)
   uint4* posg = nullptr;       // FP32 path: posq with g in .w (pass 1 -> pass 2)
   int* nbl = nullptr;          // column-major [max_nb][nmax]
@@ -179,6 +180,8 @@ struct apip_ctx {
   void* zeta = nullptr; void* xi_p = nullptr; void* e_eam = nullptr; void* g = nullptr;
   void* wbar = nullptr; void* dd = nullptr; void* lam = nullptr; void* dlam = nullptr;
   void* e_ace = nullptr;
+  void* pair_keep = nullptr;   // FP64 path: double2 [pair_rows][nmax], pass 1's pair terms for pass 2
+  int pair_rows = 0;
   double* cvec = nullptr;      // [nmax] grad-lambda CSP coefficients (kept zero between calls)
   int* ace_list = nullptr;     // [nmax]
   int* clist = nullptr;        // [nmax] learned switch: atoms with a grad-lambda coefficient

@@ -88,17 +88,33 @@ template <typename T> struct Plain {
   __device__ __forceinline__ T value() const { return s; }
 };
 
+// x < y for non-negative doubles by their bit patterns (they order as integers):
+// float64 comparisons go to the float64 pipe, two a cycle and SM.
+__device__ __forceinline__ bool less_pos(double x, double y) {
+  return (unsigned long long)__double_as_longlong(x) < (unsigned long long)__double_as_longlong(y);
+}
+
 // r = |d| and 1/r from r^2: in float32 through the reciprocal square root
-// (rsqrtf, within 2 ulp), in float64 by the correctly rounded square root and a
-// division.
+// (rsqrtf, within 2 ulp); in float64 from the hardware's approximate reciprocal
+// square root y by Newton's iteration on both (each step an exact residual by a
+// multiply-add): ten float64 operations for the two, both within one ulp, where a
+// square root and a division take some twenty.
 template <typename T> __device__ __forceinline__ void len_inv(T r2, T* r, T* ir);
 template <> __device__ __forceinline__ void len_inv<float>(float r2, float* r, float* ir) {
   *ir = rsqrtf(r2);
   *r = r2 * *ir;
 }
 template <> __device__ __forceinline__ void len_inv<double>(double r2, double* r, double* ir) {
-  *r = sqrt(r2);
-  *ir = 1.0 / *r;
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r2));
+  const double h = 0.5 * y;
+  double s = r2 * y;
+  s = fma(fma(-s, s, r2), h, s);
+  s = fma(fma(-s, s, r2), h, s);
+  y = fma(fma(-s, y, 1.0), y, y);
+  y = fma(fma(-s, y, 1.0), y, y);
+  *r = s;
+  *ir = y;
 }
 
 // Positions.  FP64 path: the caller's float64 array, minimum image with rint.
@@ -112,12 +128,21 @@ template <typename T> struct PosView;
 template <> struct PosView<double> {
   const double* pos;
   double L[3], invL[3];
+  int half_hi[3];   // high word of L / 2
   struct Self { double x, y, z; };
   using Rec = Self;   // what a neighbour's separation needs (fetch, then vec_of)
   __device__ __forceinline__ Self self(int i) const { return {pos[3 * i], pos[3 * i + 1], pos[3 * i + 2]}; }
   __device__ __forceinline__ Rec fetch(int j) const { return self(j); }
   __device__ __forceinline__ V3<double> vec_of(const Self& s, const Rec& o) const {
     double dx = o.x - s.x, dy = o.y - s.y, dz = o.z - s.z;
+    // the nearest image differs only where a component is about L / 2 or more (tested
+    // on the high words, off the float64 pipe): elsewhere rint gives 0
+    if ((__double2hiint(dx) & 0x7fffffff) >= half_hi[0] || (__double2hiint(dy) & 0x7fffffff) >= half_hi[1] ||
+        (__double2hiint(dz) & 0x7fffffff) >= half_hi[2])
+      return nearest(dx, dy, dz);
+    return {dx, dy, dz};
+  }
+  __device__ __noinline__ V3<double> nearest(double dx, double dy, double dz) const {
     dx -= L[0] * rint(dx * invL[0]);
     dy -= L[1] * rint(dy * invL[1]);
     dz -= L[2] * rint(dz * invL[2]);

@@ -50,18 +50,23 @@ struct Args {
   double r_list2, skin_half2, csp_rcut2;
   float skin_half2_f;     // skin_half2 rounded down to float (the FP32 path's rebuild trigger)
   double r_e_in2, r_e_mid2;   // list-order bounds: eam_rc^2, (eam_rc + skin + margin)^2
+  float r_e_in2f, r_e_mid2f, r_list2f;   // FP32 path: the same, and r_list^2 rounded up
+  float r_scan2f;         // the fill's first test: (r_list (1 + 2e-5))^2
+  int lanes;              // threads per atom of the list fill and the passes (atom_lanes)
+  double2* pair_keep;     // FP64 path: pass 1's EAM pair terms of the first pair_rows list entries, for pass 2
+  int pair_rows;
 
   const double* pos;      // caller positions [n][3]
   const int* id;          // caller ids [n]
   int* nnb; int* nbl; int* nbl_tmp; double* pos_ref; uint4* posq; uint4* posq_ref; int* id2idx; int* csp;
   int* csp_idx; int* csp_owner;   // CSP^list partner indices by atom index (cache), the id each row is for
   int* nnb_e;             // entries of the list whose build-time distance is below eam_rc + skin
-  int* nnb_0;             // FP32 path: entries whose build-time distance is below eam_rc
+  int* nnb_0;             // entries whose build-time distance is below eam_rc
   float* mind1;           // FP32 path: least squared build-time distance of the entries in [eam_rc, eam_rc + skin)
   uint4* posg;            // FP32 path: (posq.x, posq.y, posq.z, bits of g), written by pass 1
-  int* cell_count; int* cell_atoms;   // binning counts (zero outside a build) and members
+  int* cell_count;        // binning counts (zero outside a build)
   int ncell;
-  uint4* cell_q;          // FP32 path: fixed-point positions of the cell members, cell order
+  uint4* cell_q;          // cell members: FP32 fixed-point position, FP64 float position in the cell; index in .w
   T* zeta; T* xi_p; T* e_eam; T* g; T* wbar; T* dd; T* lam; T* dlam; T* e_ace;
   double* cvec; int* ace_list; int* counts; int* flags; int* status;
   int det;                // deterministic mode: fixed-point scatter sums, index-ordered compaction
@@ -208,6 +213,15 @@ __device__ __forceinline__ double ind_energy(const Args<T>& a, int i) {
   if (!a.ind_on) return 0.0;
   double e, f[3];
   return ind_term(a, i, &e, f) ? e : 0.0;
+}
+
+// Threads per atom of the list fill, pass 1 and pass 2.  One thread per atom makes
+// full use of the GPU only from some 150 k atoms on; below, an atom's ~60 entries
+// (~300 candidates in the fill) are shared by 4 or 8 threads as long as that still
+// leaves no SM with more than four blocks.
+inline int atom_lanes(int64_t n, int sms) {
+  const int64_t fill = (int64_t)4 * kBlock * sms;
+  return 8 * n <= fill ? 8 : (4 * n <= fill ? 4 : 1);
 }
 
 // Launch with programmatic stream serialization (the kernel must start with
