@@ -129,8 +129,8 @@ __host__ __device__ __forceinline__ int pool_elems(int n, int KA) {
 // consecutive pairs start in different banks.
 template <int LMAX>
 __host__ __device__ constexpr int ry_stride() { return (kNmaxCap + (LMAX + 1) * (LMAX + 1)) | 1; }
-template <int LMAX>
-__host__ __device__ constexpr int ry_elems() { return kAceThreads * ry_stride<LMAX>(); }
+template <int LMAX, int NT = kAceThreads>
+__host__ __device__ constexpr int ry_elems() { return NT * ry_stride<LMAX>(); }
 
 // Per-atom state of a group, in static shared memory.
 template <typename T, int NAT>
@@ -195,13 +195,13 @@ __device__ __forceinline__ void group_setup(const Args<T>& a, int grp, int count
 // float-float; then d, lam = 1 - f_trans(d) and dlam in float64 (a few operations
 // per atom).  The results replace the atom's lam, dlam, w-bar and d (read by
 // atom_scalars).  Ends with a barrier.
-template <typename T, int NAT>
+template <typename T, int NAT, int NT = kAceThreads>
 __device__ __forceinline__ void refine_switch(const Args<T>& a, const AceGroup<T, NAT>& g) {
   if constexpr (sizeof(T) == 4) {
     if (a.lam_mode == APIP_LAM_PAPER || a.lam_mode == APIP_LAM_LEARNED) {
       const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
       const SwFF& sw = a.swff;
-      for (int k = warp; k < NAT; k += kAceWarps) {
+      for (int k = warp; k < NAT; k += NT / 32) {
         const int i = g.atom[k];
         if (i < 0 || a.dlam[i] == T(0)) continue;   // not transitional (constant-lam atoms: dlam = 0)
         const uint4 qi = a.pv.q[i];
@@ -269,12 +269,12 @@ __device__ __forceinline__ void refine_switch(const Args<T>& a, const AceGroup<T
 }
 
 // Step 1: A[c * NAT + k] += a_scale sum_j R Y (A zeroed by the caller; RY is a
-// staging area of ry_elems<LMAX>() elements).  The pairs are taken 256 at a
-// time; after their R, Y rows are staged, the (atom, component) sums are formed
+// staging area of ry_elems<LMAX, NT>() elements).  The pairs are taken NT (the
+// block) at a time; after their R, Y rows are staged, the (atom, component) sums are formed
 // only for the atoms that have pairs in that chunk, the components of one atom
 // on consecutive threads (which then read the same staged rows).  Ends with a
 // barrier.
-template <typename T, typename K, int LMAX, int NAT>
+template <typename T, typename K, int LMAX, int NAT, int NT = kAceThreads>
 __device__ __forceinline__ void densities(const Args<T>& a, const AceDev<T>& t, const AceGroup<T, NAT>& g,
                                           T* A, T* RY) {
   constexpr int NLM = (LMAX + 1) * (LMAX + 1);
@@ -283,7 +283,7 @@ __device__ __forceinline__ void densities(const Args<T>& a, const AceDev<T>& t, 
   const int nA = t.nA;
   const T rc2 = t.rc * t.rc;
   const int total = g.off[NAT];
-  for (int base = 0; base < total; base += kAceThreads) {
+  for (int base = 0; base < total; base += NT) {
     const int p = base + tid;
     T* ry = RY + tid * RYS;
     bool in = false;
@@ -311,10 +311,10 @@ __device__ __forceinline__ void densities(const Args<T>& a, const AceDev<T>& t, 
       for (int q = 0; q < RYS; ++q) ry[q] = T(0);
     }
     __syncthreads();
-    const int hp = min(total - base, kAceThreads);
+    const int hp = min(total - base, NT);
     const int k0 = atom_of_pair<NAT>(base, g.off), k1 = atom_of_pair<NAT>(base + hp - 1, g.off);
     const int items = nA * (k1 - k0 + 1);
-    for (int item = tid; item < items; item += kAceThreads) {
+    for (int item = tid; item < items; item += NT) {
       const int k = k0 + item / nA, c = item - (k - k0) * nA;
       const int n = c / NLM, lm = c - n * NLM;
       const int lo = max(g.off[k] - base, 0), hi = min(g.off[k + 1] - base, hp);
@@ -324,7 +324,7 @@ __device__ __forceinline__ void densities(const Args<T>& a, const AceDev<T>& t, 
     }
     __syncthreads();
   }
-  for (int item = tid; item < nA * NAT; item += kAceThreads) A[item] *= t.a_scale;
+  for (int item = tid; item < nA * NAT; item += NT) A[item] *= t.a_scale;
   __syncthreads();
 }
 
@@ -357,7 +357,7 @@ __device__ __forceinline__ void atom_scalars(const Args<T>& a, const AceDev<T>& 
 
 // Step 4 with omega W[c * NAT + k], then the per-atom energies; returns this
 // thread's energy contribution (non-zero only for tid < NAT).  Ends with a barrier.
-template <typename T, typename K, int LMAX, int NAT>
+template <typename T, typename K, int LMAX, int NAT, int NT = kAceThreads>
 __device__ __forceinline__ double pair_forces(const Args<T>& a, const AceDev<T>& t, const AceGroup<T, NAT>& g,
                                               const T* W) {
   constexpr int NLM = (LMAX + 1) * (LMAX + 1);
@@ -369,7 +369,7 @@ __device__ __forceinline__ double pair_forces(const Args<T>& a, const AceDev<T>&
   const bool eam_corr = !a.precise_adds_eam && a.eam_force && !a.force_mix;
   const int n_max = t.n_max;
   const int total = g.off[NAT];
-  for (int base = 0; base < total; base += kAceThreads) {
+  for (int base = 0; base < total; base += NT) {
     const int p = base + tid;
     if (p >= total) continue;
     const int k = atom_of_pair<NAT>(p, g.off);

@@ -349,6 +349,160 @@ void gaunt_fill(double* out) {
       }
 }
 
+void gaunt4_fill(double* out) {
+  for (int l1 = 0; l1 <= kGauntLmax; ++l1)
+    for (int l2 = l1; l2 <= kGauntLmax; ++l2)
+      for (int L = l2 - l1; L <= l1 + l2; L += 2) {
+        int e = gaunt4_offset(l1, l2, L);
+        for (int m1 = -l1; m1 <= l1; ++m1)
+          for (int m2 = -l2; m2 <= l2; ++m2)
+            for (int v = 0; v < 2; ++v) {
+              const int M = gaunt_cand(m1, m2, v, L);
+              if (M != kNoM) out[e++] = real_gaunt(l1, m1, l2, m2, L, M);
+            }
+      }
+}
+
+// Quadratic tables (body order 4, float32).  The rows of X_L are the couplings
+// C_{(p q) L} (p <= q) that some function uses, then the segments A_{n L}, then (L = 0)
+// the constant 1; a function of degree L is the product of two rows.  S_L holds the
+// coefficients of both channels symmetrically (a square twice), K2_L those of
+// channel 2 once.  The function order p <= q <= s <= u leaves two thirds of S_L
+// empty, so a tile of kQuadTile rows keeps only the columns that one of its rows
+// has; with the rows ordered by (n_q, p) the tiles of an 8 / 4 basis hold 1.33 times
+// the entries that are there (ordered by (p, q) 1.68 times).  Tiles are listed by
+// falling length.
+bool build_quad(int n_max, int l_max, const double* c1, const double* c2, int64_t n_basis, HostQuad* out,
+                std::string* err) {
+  const auto basis = enumerate(n_max, l_max, 4);
+  if ((int64_t)basis.size() != n_basis) { *err = "ace_n_basis does not match the canonical basis size"; return false; }
+  auto pid = [&](int n, int l) { return (n - 1) * (l_max + 1) + l; };
+  auto nq = [&](int p) { return p / (l_max + 1) + 1; };
+  auto lq = [&](int p) { return p % (l_max + 1); };
+  typedef std::array<int, 2> Slot;   // (p, q); (-1, n) = A_{n L}; (-2, 0) = 1
+  struct Fn { Slot x, y; double a, b; };
+  std::vector<std::vector<Fn>> fn(kQuadLs);
+  for (size_t k = 0; k < basis.size(); ++k) {
+    const Basis& b = basis[k];
+    int p[4];
+    for (int q = 0; q < b.nu; ++q) p[q] = pid(b.n[q], b.l[q]);
+    Fn f{{-1, b.n[0]}, {-2, 0}, c1[k], c2[k]};
+    int L = 0;
+    if (b.nu == 2) { L = b.l[0]; f.y = {-1, b.n[1]}; }
+    else if (b.nu == 3) { L = b.l[2]; f.x = {p[0], p[1]}; f.y = {-1, b.n[2]}; }
+    else if (b.nu == 4) { L = b.L; f.x = {p[0], p[1]}; f.y = {p[2], p[3]}; }
+    fn[L].push_back(f);
+  }
+  out->hdr.assign(4 * kQuadLs, 0);
+  out->map.assign((size_t)kQuadLs * kQuadMap, -1);
+  out->tile.clear(); out->val.clear(); out->col.clear();
+  out->rows = 0;
+  for (int L = 0; L <= 2 * l_max; ++L) {
+    const int step = (2 * L + 1) * kQuadAtoms;
+    std::map<Slot, int> row;
+    std::vector<Slot> slots;
+    for (const Fn& f : fn[L])
+      for (const Slot& s : {f.x, f.y})
+        if (s[0] >= 0 && row.emplace(s, 0).second) slots.push_back(s);
+    std::sort(slots.begin(), slots.end(), [&](const Slot& x, const Slot& y) {
+      return std::make_tuple(nq(x[1]), x[0], x[1]) < std::make_tuple(nq(y[1]), y[0], y[1]);
+    });
+    const int nc = (int)slots.size(), na = L <= l_max ? n_max : 0;
+    for (int k = 0; k < nc; ++k) {
+      row[slots[k]] = k;
+      const int p = slots[k][0], q = slots[k][1];
+      short* m = out->map.data() + (size_t)L * kQuadMap;
+      auto at = [&](int u, int v) { return ((lq(u) * (kLmaxCap + 1) + lq(v)) * kNmaxCap + nq(u) - 1) * kNmaxCap + nq(v) - 1; };
+      m[at(p, q)] = m[at(q, p)] = (short)k;
+    }
+    for (int n = 1; n <= na; ++n) row[Slot{-1, n}] = nc + n - 1;
+    if (L == 0) row[Slot{-2, 0}] = nc + na;
+    const int nr = nc + na + (L == 0 ? 1 : 0);
+    std::vector<double> s1((size_t)nr * nr, 0.0), s2(s1), k2(s1);
+    for (const Fn& f : fn[L]) {
+      const size_t x = row[f.x], y = row[f.y];
+      s1[x * nr + y] += f.a; s1[y * nr + x] += f.a;
+      s2[x * nr + y] += f.b; s2[y * nr + x] += f.b;
+      k2[x * nr + y] += f.b;
+    }
+    struct Tile { int rec[8]; };
+    std::vector<Tile> tiles;
+    for (int r0 = 0; r0 < nr; r0 += kQuadTile) {
+      const int r1 = std::min(nr, r0 + kQuadTile);
+      Tile t{};
+      for (int pass = 0; pass < 2; ++pass) {   // S (both channels), K2
+        std::vector<int> cols;
+        for (int c = 0; c < nr; ++c) {
+          bool any = false;
+          for (int r = r0; r < r1; ++r) {
+            const size_t e = (size_t)r * nr + c;
+            any = any || (pass == 0 ? s1[e] != 0.0 || s2[e] != 0.0 : k2[e] != 0.0);
+          }
+          if (any) cols.push_back(c);
+        }
+        const size_t unit = pass == 0 ? 2 : 4;   // columns per 128 bytes of values
+        while (cols.size() % unit) cols.push_back(-1);
+        t.rec[4 * pass] = (int)(out->val.size() / 4);
+        t.rec[4 * pass + 1] = (int)out->col.size();
+        t.rec[4 * pass + 2] = (int)cols.size();
+        for (int c : cols) {
+          out->col.push_back(c < 0 ? 0u : (uint32_t)(c * step));
+          for (int r = r0; r < r0 + kQuadTile; ++r) {
+            const bool in = c >= 0 && r < r1;
+            const size_t e = (size_t)r * nr + c;
+            if (pass == 0) {
+              out->val.push_back(in ? (float)s1[e] : 0.f);
+              out->val.push_back(in ? (float)s2[e] : 0.f);
+            } else {
+              out->val.push_back(in ? (float)k2[e] : 0.f);
+            }
+          }
+        }
+        while (out->col.size() % 4) out->col.push_back(0u);
+      }
+      t.rec[3] = r0;
+      t.rec[7] = r1 - r0;
+      tiles.push_back(t);
+    }
+    std::stable_sort(tiles.begin(), tiles.end(), [](const Tile& x, const Tile& y) { return x.rec[2] > y.rec[2]; });
+    const int hdr[4] = {nc, na, (int)out->tile.size() / 8, (int)tiles.size()};
+    std::copy(hdr, hdr + 4, out->hdr.begin() + 4 * L);
+    for (const Tile& t : tiles) out->tile.insert(out->tile.end(), t.rec, t.rec + 8);
+    out->rows = std::max(out->rows, nr * (2 * L + 1));
+  }
+  // the loops read one step past a tile's last
+  out->val.insert(out->val.end(), 32, 0.f);
+  out->col.insert(out->col.end(), 4, 0u);
+  return true;
+}
+
+// Every offset of the quadratic tables lies within its array.
+bool validate_quad(const HostQuad& h, std::string* err) {
+  auto bad = [&](const std::string& what) { *err = "internal: ACE table check failed: " + what; return false; };
+  if (h.hdr.size() != 4 * kQuadLs || h.map.size() != (size_t)kQuadLs * kQuadMap) return bad("degree tables");
+  for (int L = 0; L < kQuadLs; ++L) {
+    const int nc = h.hdr[4 * L], na = h.hdr[4 * L + 1], t0 = h.hdr[4 * L + 2], nt = h.hdr[4 * L + 3];
+    const int nr = nc + na + (L == 0 ? 1 : 0), step = (2 * L + 1) * kQuadAtoms;
+    if (nc < 0 || na < 0 || nr * (2 * L + 1) > h.rows || t0 < 0 || (size_t)8 * (t0 + nt) > h.tile.size())
+      return bad("degree " + std::to_string(L));
+    for (int k = 0; k < kQuadMap; ++k)
+      if (h.map[(size_t)L * kQuadMap + k] < -1 || h.map[(size_t)L * kQuadMap + k] >= nc) return bad("row map");
+    for (int t = t0; t < t0 + nt; ++t) {
+      const int* r = h.tile.data() + 8 * t;
+      if (r[3] < 0 || r[7] < 1 || r[7] > kQuadTile || r[3] + r[7] > nr) return bad("tile rows");
+      for (int pass = 0; pass < 2; ++pass) {
+        const int v = r[4 * pass], c = r[4 * pass + 1], n = r[4 * pass + 2], unit = pass == 0 ? 2 : 4;
+        if (n < 0 || n % unit || v < 0 || v % 8 || c < 0 || c % 4) return bad("tile alignment");
+        if ((size_t)4 * v + (size_t)n * 32 / unit + 32 > h.val.size() || (size_t)c + n + 4 > h.col.size())
+          return bad("tile extent");
+        for (int k = c; k < c + n; ++k)
+          if (h.col[k] % step || (int)(h.col[k] / step) >= nr) return bad("tile column");
+      }
+    }
+  }
+  return true;
+}
+
 // Streamed tables (body order <= 3): couplings C_{(p1 p2) L} with l1 <= l2 (the
 // factors swapped where needed; C is symmetric in them), sorted by type so that
 // neighbouring thread slices run the same unrolled code, each with its list of

@@ -345,6 +345,16 @@ AceDev<T> ace_dev(apip_ctx* c) {
     t.group = c->ace_group;
     return t;
   }
+  if (t.kind == kAceQuad) {
+    t.qhdr = reinterpret_cast<const int4*>(b + c->ace_off[0]);
+    t.qmap = reinterpret_cast<const short*>(b + c->ace_off[1]);
+    t.qtile = reinterpret_cast<const int4*>(b + c->ace_off[2]);
+    t.qval = reinterpret_cast<const ulonglong2*>(b + c->ace_off[3]);
+    t.qcol = reinterpret_cast<const uint32_t*>(b + c->ace_off[4]);
+    t.qrows = c->ace_qrows;
+    t.group = c->ace_group;
+    return t;
+  }
   t.comp = reinterpret_cast<const uint2*>(b + c->ace_off[0]);
   t.gent = reinterpret_cast<const Ent<T>*>(b + c->ace_off[1]);
   t.frec = reinterpret_cast<const Rec<T>*>(b + c->ace_off[2]);
@@ -399,7 +409,10 @@ void force_pipeline(apip_ctx* c, Args<T>& a, cudaStream_t s) {
     if (a.force_mix) launch_fm_buffer<T>(a, s); }
   { NvtxRange nv("apip.ace"); Phase ph(c, APIP_PHASE_ACE, 1, s); const AceDev<T> t = ace_dev<T>(c);
     if (t.kind == kAceStreamed) launch_ace_stream<T>(a, t, c->ace_blocks, s);
-    else launch_ace_pool<T>(a, t, c->ace_blocks, s); }
+    else if constexpr (sizeof(T) == 4) {
+      if (t.kind == kAceQuad) launch_ace_quad(a, t, c->ace_blocks, s);
+      else launch_ace_pool<T>(a, t, c->ace_blocks, s);
+    } else launch_ace_pool<T>(a, t, c->ace_blocks, s); }
   if (a.lam_mode == APIP_LAM_PAPER && a.grad_lambda) {
     NvtxRange nv("apip.csp");
     Phase ph(c, APIP_PHASE_CSP, 1, s);
@@ -529,8 +542,12 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
   ctx->p.ace_c2 = nullptr;
   ctx->nmax = n_atoms_max;
   ctx->r_list = std::max(std::max(p->eam_rc, p->ace_rc), p->sw_r_w) + p->skin;
-  // body order <= 3: streamed couplings; body order 4: the coupling pool
+  // body order <= 3: streamed couplings; body order 4: in float32 the quadratic
+  // evaluation, which has its own atoms per block, in float64 or with a group size
+  // asked for the coupling pool
   const bool streamed = p->ace_nu_max <= 3;
+  const bool quad = !streamed && p->precision == APIP_FP32 && p->ace_group == 0;
+  HostQuad hq;
   HostAce tab;
   HostStream st;
   if (streamed ? !build_streamed(p->ace_n_max, p->ace_l_max, p->ace_nu_max, ctx->ace_c1.data(), ctx->ace_c2.data(),
@@ -545,7 +562,12 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
     delete ctx;
     return APIP_ERR_ARG;
   }
-  ctx->ace_kind = streamed ? kAceStreamed : kAcePool;
+  if (quad && !(build_quad(p->ace_n_max, p->ace_l_max, ctx->ace_c1.data(), ctx->ace_c2.data(), nb, &hq, &why) &&
+                validate_quad(hq, &why))) {
+    delete ctx;
+    return APIP_ERR_ARG;
+  }
+  ctx->ace_kind = streamed ? kAceStreamed : (quad ? kAceQuad : kAcePool);
   const int nA = p->ace_n_max * (p->ace_l_max + 1) * (p->ace_l_max + 1);
   auto fail_create = [&](cudaError_t e) {
     free_all(ctx);
@@ -581,7 +603,12 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
       return streamed ? ace_stream_occupancy<double>(t) : ace_pool_occupancy<double>(t);
     };
     int group = p->ace_group, occ = 0;
-    if (group != 0) {
+    if (quad) {
+      AceDev<float> t{};
+      t.l_max = p->ace_l_max; t.nA = nA; t.qrows = hq.rows;
+      group = kQuadAtoms;
+      occ = ace_quad_occupancy(t);
+    } else if (group != 0) {
       occ = occ_of(group);   // 0 for a group the kernel does not provide
     } else if (streamed) {
       const bool adaptive = p->lam_mode == APIP_LAM_PAPER || p->lam_mode == APIP_LAM_LEARNED;
@@ -735,6 +762,14 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
     info[10] = 11 * st.gaunt_products + 6 * part_len + 6 * (int64_t)st.tkey.size() + 6 * pair_len +
                6 * (int64_t)st.pkey.size();
   } else {
+    if (quad) {
+      put(0, hq.hdr.data(), sizeof(int) * hq.hdr.size());
+      put(1, hq.map.data(), sizeof(short) * hq.map.size());
+      put(2, hq.tile.data(), sizeof(int) * hq.tile.size());
+      put(3, hq.val.data(), sizeof(float) * hq.val.size());
+      put(4, hq.col.data(), sizeof(uint32_t) * hq.col.size());
+      ctx->ace_qrows = hq.rows;
+    } else {
     put(0, tab.comp.data(), sizeof(uint32_t) * tab.comp.size());
     put_ent(1, tab.gkey, tab.gval);
     put_rec(2, tab.fkey, &tab.flen, tab.f1, tab.f2);
@@ -743,6 +778,7 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
     put_ent(5, tab.bkey, tab.bval);
     put(6, tab.poff.data(), sizeof(int) * tab.poff.size());
     put(7, tab.tpiece.data(), sizeof(int) * tab.tpiece.size());
+    }
     ctx->ace_nC = tab.nC;
     ctx->ace_npool = tab.npool;
     ctx->ace_nf = (int)tab.fkey.size();
@@ -761,7 +797,7 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
   }
   ctx->ace_info[7] = ctx->ace_group;
   ctx->ace_info[8] = ctx->ace_blocks;
-  ctx->ace_info[9] = ctx->ace_kind;
+  ctx->ace_info[9] = streamed ? 1 : 0;
   APIP_ALLOC(ctx->ace_tab, host.size());
 #undef APIP_ALLOC
   cudaError_t e = cudaMemcpy(ctx->ace_tab, host.data(), host.size(), cudaMemcpyHostToDevice);
@@ -789,6 +825,8 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
     gaunt_fill(gv.data());
     e = p->precision == APIP_FP64 ? ace_stream_set_consts<double>(norms, nn, gv.data())
                                   : ace_stream_set_consts<float>(norms, nn, gv.data());
+  } else if (quad) {
+    e = ace_quad_set_consts(norms, nn);
   } else {
     e = p->precision == APIP_FP64 ? ace_pool_set_norms<double>(norms, nn) : ace_pool_set_norms<float>(norms, nn);
   }

@@ -79,7 +79,16 @@ template <typename T> struct alignas(sizeof(T) == 4 ? 8 : 16) Ent { T v; uint32_
 //  streamed (body order <= 3, built by build_streamed): the couplings are formed
 //    one at a time in registers and contracted with their nu = 3 partners; nu = 1, 2
 //    functions are dot products of A segments.
-constexpr int kAcePool = 0, kAceStreamed = 1;
+//  quadratic (body order 4 in float32, built by build_quad): the couplings of one
+//    degree L and the A segments of that degree are the rows of a matrix X_L, and
+//    every function of that degree is an entry of a symmetric matrix S_L shared by
+//    all atoms: phi_c = sum_L 1/2 X_L . (S_L^c X_L).
+constexpr int kAcePool = 0, kAceStreamed = 1, kAceQuad = 2;
+constexpr int kQuadAtoms = 8;       // atoms per block of the quadratic evaluation
+constexpr int kQuadThreads = 384;   // its threads per block
+constexpr int kQuadTile = 8;        // rows of S_L per tile
+constexpr int kQuadLs = 2 * kLmaxCap + 1;                       // degrees L of a coupling
+constexpr int kQuadMap = (kLmaxCap + 1) * (kLmaxCap + 1) * kNmaxCap * kNmaxCap;   // rowmap entries per degree
 
 template <typename T>
 struct AceDev {
@@ -100,6 +109,13 @@ struct AceDev {
   const uint4* cpl; int ncpl;   // couplings: (a1 | a2 << 8 | type << 16, partner begin, partner end, 0)
   const Rec<T>* part; int npart;  // nu = 3 partners: key = A index of A_{p3, m = -l3}
   const Rec<T>* cfirst;         // the first partner record of each coupling (a copy, loaded with the coupling)
+  // quadratic tables
+  const int4* qhdr;             // [kQuadLs] (C rows, A rows, first tile, tiles)
+  const short* qmap;            // [kQuadLs][l1][l2][n1 - 1][n2 - 1]: row of C_{(n1 l1)(n2 l2) L}, -1: none
+  const int4* qtile;            // [2 tiles] (S values / 16 bytes, column list, columns, first row) of S, (.., rows) of K2
+  const ulonglong2* qval;       // values
+  const uint32_t* qcol;         // columns as offsets of their rows in X_L
+  int qrows;                    // most values of X_L per atom
   int group;                    // compacted atoms per thread block
 };
 
@@ -121,12 +137,26 @@ struct HostAce {
   std::vector<int> poff, tpiece;
 };
 
+// Tables of the quadratic evaluation (fields as in AceDev).
+struct HostQuad {
+  std::vector<int> hdr;               // [4 kQuadLs]
+  std::vector<short> map;             // [kQuadLs kQuadMap]
+  std::vector<int> tile;              // [8 per tile]
+  std::vector<float> val;
+  std::vector<uint32_t> col;
+  int rows = 0;
+};
+
 // ace_tables.cpp
 int64_t basis_size(int n_max, int l_max, int nu_max);
 bool build_coupled(int n_max, int l_max, int nu_max, const double* c1, const double* c2, int64_t n_basis,
                    HostAce* out, std::string* err);
 bool build_streamed(int n_max, int l_max, int nu_max, const double* c1, const double* c2, int64_t n_basis,
                     HostStream* out, std::string* err);
+bool build_quad(int n_max, int l_max, const double* c1, const double* c2, int64_t n_basis, HostQuad* out,
+                std::string* err);
+bool validate_quad(const HostQuad& h, std::string* err);
+void gaunt4_fill(double* out);   // kGaunt4Total entries
 bool validate_streamed(const HostStream& h, int nA, std::string* err);
 bool validate_coupled(const HostAce& h, std::string* err);
 // real Gaunt values in the canonical layout of gaunt_layout.h (kGauntTotal entries)
@@ -208,6 +238,7 @@ struct apip_ctx {
   // the byte offsets ace_off (order of AceDev's pointers)
   void* ace_tab = nullptr;
   size_t ace_off[8] = {};
+  int ace_qrows = 0;
   int ace_nf = 0, ace_npc = 0, ace_nC = 0, ace_npool = 0;
   int ace_group = 1;
   int ace_kind = 0, ace_npr = 0, ace_ncpl = 0, ace_npart = 0;

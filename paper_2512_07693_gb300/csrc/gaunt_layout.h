@@ -69,4 +69,30 @@ __host__ __device__ constexpr int gaunt_type(int l1, int l2, int L) { return (l1
   X(1, 3, 2) X(1, 3, 4) X(1, 4, 3) X(2, 2, 0) X(2, 2, 2) X(2, 2, 4) X(2, 3, 1) X(2, 3, 3) X(2, 4, 2)          \
   X(2, 4, 4) X(3, 3, 0) X(3, 3, 2) X(3, 3, 4) X(3, 4, 1) X(3, 4, 3) X(4, 4, 0) X(4, 4, 2) X(4, 4, 4)
 
+// The same for the couplings of body order 4, whose degree L goes up to 2 l_max:
+// offset of type (l1 <= l2, L <= 8), past the last type the table size.
+constexpr int kGaunt4L = 2 * kGauntLmax;
+__host__ __device__ constexpr int gaunt4_offset(int l1, int l2, int L) {
+  int off = 0;
+  for (int x = 0; x <= kGauntLmax; ++x)
+    for (int y = x; y <= kGauntLmax; ++y)
+      for (int z = y - x; z <= x + y; z += 2) {
+        if (x == l1 && y == l2 && z == L) return off;
+        off += gaunt_count(x, y, z);
+      }
+  return off;
+}
+constexpr int kGaunt4Total = gaunt4_offset(kGauntLmax + 1, 0, 0);
+
+// every (l1 <= l2 <= 4) that couples to degree L, by L
+#define APIP_GAUNT4_L0(X) X(0, 0, 0) X(1, 1, 0) X(2, 2, 0) X(3, 3, 0) X(4, 4, 0)
+#define APIP_GAUNT4_L1(X) X(0, 1, 1) X(1, 2, 1) X(2, 3, 1) X(3, 4, 1)
+#define APIP_GAUNT4_L2(X) X(0, 2, 2) X(1, 1, 2) X(1, 3, 2) X(2, 2, 2) X(2, 4, 2) X(3, 3, 2) X(4, 4, 2)
+#define APIP_GAUNT4_L3(X) X(0, 3, 3) X(1, 2, 3) X(1, 4, 3) X(2, 3, 3) X(3, 4, 3)
+#define APIP_GAUNT4_L4(X) X(0, 4, 4) X(1, 3, 4) X(2, 2, 4) X(2, 4, 4) X(3, 3, 4) X(4, 4, 4)
+#define APIP_GAUNT4_L5(X) X(1, 4, 5) X(2, 3, 5) X(3, 4, 5)
+#define APIP_GAUNT4_L6(X) X(2, 4, 6) X(3, 3, 6) X(4, 4, 6)
+#define APIP_GAUNT4_L7(X) X(3, 4, 7)
+#define APIP_GAUNT4_L8(X) X(4, 4, 8)
+
 }  // namespace apip

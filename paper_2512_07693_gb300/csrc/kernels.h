@@ -299,6 +299,10 @@ void launch_mlp_adam(float* p, const float* g, float* m, float* v, int t, float 
 template <typename T> cudaError_t ace_pool_set_norms(const double* norms, int count);
 template <typename T> void launch_ace_pool(const Args<T>& a, const AceDev<T>& ace, int blocks, cudaStream_t s);
 template <typename T> int ace_pool_occupancy(const AceDev<T>& ace);
+// the quadratic evaluation of body order 4 in float32 (kernels_ace4_f32.cu)
+cudaError_t ace_quad_set_consts(const double* norms, int count);
+void launch_ace_quad(const Args<float>& a, const AceDev<float>& ace, int blocks, cudaStream_t s);
+int ace_quad_occupancy(const AceDev<float>& ace);
 template <typename T> cudaError_t ace_stream_set_consts(const double* norms, int count, const double* gaunt);
 template <typename T> void launch_ace_stream(const Args<T>& a, const AceDev<T>& ace, int blocks, cudaStream_t s);
 template <typename T> int ace_stream_occupancy(const AceDev<T>& ace);
