@@ -109,34 +109,34 @@ __device__ __forceinline__ void quad_back(const float* A, const float* Y, const 
 
 // acc[r][j] += value(r) . X(column, j) over the columns of a tile; F2 rows are the two
 // channels of one row of S (NP = 8) or two rows of K2 (NP = 4).  The values of the
-// next 128 bytes and their columns are loaded while these are used.
+// next step (2 or 4 columns) and their columns are loaded while these are used.
 template <int NP>
 __device__ __forceinline__ void quad_tile(const ulonglong2* val, const uint32_t* col, int len, const float* Xq,
                                           F2 (&acc)[NP][4]) {
-  constexpr int U = 16 / NP;   // columns per 128 bytes
+  constexpr int U = 16 / NP;   // columns per step (128 bytes of values)
   ulonglong2 vn[8];
   uint32_t cn[U];
-  auto fetch = [&](int s) {
+  auto fetch = [&](int st) {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) vn[q] = __ldg(val + (size_t)s / U * 8 + q);
+    for (int q = 0; q < 8; ++q) vn[q] = __ldg(val + (size_t)(st * 8 + q) * kQuadBundle);
     if constexpr (U == 2) {
-      const uint2 c = __ldg(reinterpret_cast<const uint2*>(col + s));
+      const uint2 c = __ldg(reinterpret_cast<const uint2*>(col + (size_t)st * kQuadBundle * U));
       cn[0] = c.x; cn[1] = c.y;
     } else {
-      const uint4 c = __ldg(reinterpret_cast<const uint4*>(col + s));
+      const uint4 c = __ldg(reinterpret_cast<const uint4*>(col + (size_t)st * kQuadBundle * U));
       cn[0] = c.x; cn[1] = c.y; cn[2] = c.z; cn[3] = c.w;
     }
   };
   fetch(0);
 #pragma unroll 1
-  for (int s = 0; s < len; s += U) {
+  for (int st = 0; st < len / U; ++st) {
     ulonglong2 v[8];
     uint32_t c[U];
 #pragma unroll
     for (int q = 0; q < 8; ++q) v[q] = vn[q];
 #pragma unroll
     for (int u = 0; u < U; ++u) c[u] = cn[u];
-    fetch(s + U);
+    fetch(st + 1);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const float4 x = *reinterpret_cast<const float4*>(Xq + c[u]);

@@ -371,7 +371,8 @@ void gaunt4_fill(double* out) {
 // empty, so a tile of kQuadTile rows keeps only the columns that one of its rows
 // has; with the rows ordered by (n_q, p) the tiles of an 8 / 4 basis hold 1.33 times
 // the entries that are there (ordered by (p, q) 1.68 times).  Tiles are listed by
-// falling length.
+// falling length; the values of kQuadBundle of them are interleaved 16 bytes at a time,
+// so that the lanes of a warp, which work on up to that many tiles, read one line.
 bool build_quad(int n_max, int l_max, const double* c1, const double* c2, int64_t n_basis, HostQuad* out,
                 std::string* err) {
   const auto basis = enumerate(n_max, l_max, 4);
@@ -425,54 +426,73 @@ bool build_quad(int n_max, int l_max, const double* c1, const double* c2, int64_
       s2[x * nr + y] += f.b; s2[y * nr + x] += f.b;
       k2[x * nr + y] += f.b;
     }
-    struct Tile { int rec[8]; };
+    struct Tile { int row, rows; std::vector<int> cols[2]; };   // columns of S (both channels), of K2
     std::vector<Tile> tiles;
     for (int r0 = 0; r0 < nr; r0 += kQuadTile) {
-      const int r1 = std::min(nr, r0 + kQuadTile);
-      Tile t{};
-      for (int pass = 0; pass < 2; ++pass) {   // S (both channels), K2
-        std::vector<int> cols;
+      Tile t;
+      t.row = r0;
+      t.rows = std::min(kQuadTile, nr - r0);
+      for (int pass = 0; pass < 2; ++pass) {
         for (int c = 0; c < nr; ++c) {
           bool any = false;
-          for (int r = r0; r < r1; ++r) {
+          for (int r = r0; r < r0 + t.rows; ++r) {
             const size_t e = (size_t)r * nr + c;
             any = any || (pass == 0 ? s1[e] != 0.0 || s2[e] != 0.0 : k2[e] != 0.0);
           }
-          if (any) cols.push_back(c);
+          if (any) t.cols[pass].push_back(c);
         }
         const size_t unit = pass == 0 ? 2 : 4;   // columns per 128 bytes of values
-        while (cols.size() % unit) cols.push_back(-1);
-        t.rec[4 * pass] = (int)(out->val.size() / 4);
-        t.rec[4 * pass + 1] = (int)out->col.size();
-        t.rec[4 * pass + 2] = (int)cols.size();
-        for (int c : cols) {
-          out->col.push_back(c < 0 ? 0u : (uint32_t)(c * step));
-          for (int r = r0; r < r0 + kQuadTile; ++r) {
-            const bool in = c >= 0 && r < r1;
-            const size_t e = (size_t)r * nr + c;
-            if (pass == 0) {
-              out->val.push_back(in ? (float)s1[e] : 0.f);
-              out->val.push_back(in ? (float)s2[e] : 0.f);
-            } else {
-              out->val.push_back(in ? (float)k2[e] : 0.f);
+        while (t.cols[pass].size() % unit) t.cols[pass].push_back(-1);
+      }
+      tiles.push_back(t);
+    }
+    std::stable_sort(tiles.begin(), tiles.end(),
+                     [](const Tile& x, const Tile& y) { return x.cols[0].size() > y.cols[0].size(); });
+    const int tile0 = (int)out->tile.size() / 8;
+    for (size_t b = 0; b < tiles.size(); b += kQuadBundle) {
+      const size_t nb = std::min<size_t>(kQuadBundle, tiles.size() - b);
+      int rec[kQuadBundle][8] = {};
+      for (int pass = 0; pass < 2; ++pass) {
+        const size_t unit = pass == 0 ? 2 : 4;
+        size_t len = 0;
+        for (size_t k = 0; k < nb; ++k) len = std::max(len, tiles[b + k].cols[pass].size());
+        const size_t v0 = out->val.size(), k0 = out->col.size();
+        out->val.resize(v0 + len / unit * 32 * kQuadBundle, 0.f);
+        out->col.resize(k0 + len * kQuadBundle, 0u);
+        for (size_t k = 0; k < nb; ++k) {
+          const Tile& t = tiles[b + k];
+          rec[k][4 * pass] = (int)(v0 / 4 + k);
+          rec[k][4 * pass + 1] = (int)(k0 + k * unit);
+          rec[k][4 * pass + 2] = (int)t.cols[pass].size();
+          for (size_t q = 0; q < t.cols[pass].size(); ++q) {
+            const int c = t.cols[pass][q];
+            if (c < 0) continue;
+            const size_t step_i = q / unit, u = q % unit;
+            out->col[k0 + (step_i * kQuadBundle + k) * unit + u] = (uint32_t)(c * step);
+            for (int r = 0; r < t.rows; ++r) {
+              const size_t e = (size_t)(t.row + r) * nr + c;
+              for (int ch = 0; ch < (pass == 0 ? 2 : 1); ++ch) {
+                const size_t f = pass == 0 ? u * 16 + 2 * r + ch : u * 8 + r;   // of the 32 values of this tile and step
+                out->val[v0 + ((step_i * 8 + f / 4) * kQuadBundle + k) * 4 + f % 4] =
+                    (float)(pass == 1 ? k2[e] : ch == 0 ? s1[e] : s2[e]);
+              }
             }
           }
         }
-        while (out->col.size() % 4) out->col.push_back(0u);
       }
-      t.rec[3] = r0;
-      t.rec[7] = r1 - r0;
-      tiles.push_back(t);
+      for (size_t k = 0; k < nb; ++k) {
+        rec[k][3] = tiles[b + k].row;
+        rec[k][7] = tiles[b + k].rows;
+        out->tile.insert(out->tile.end(), rec[k], rec[k] + 8);
+      }
     }
-    std::stable_sort(tiles.begin(), tiles.end(), [](const Tile& x, const Tile& y) { return x.rec[2] > y.rec[2]; });
-    const int hdr[4] = {nc, na, (int)out->tile.size() / 8, (int)tiles.size()};
+    const int hdr[4] = {nc, na, tile0, (int)tiles.size()};
     std::copy(hdr, hdr + 4, out->hdr.begin() + 4 * L);
-    for (const Tile& t : tiles) out->tile.insert(out->tile.end(), t.rec, t.rec + 8);
     out->rows = std::max(out->rows, nr * (2 * L + 1));
   }
   // the loops read one step past a tile's last
-  out->val.insert(out->val.end(), 32, 0.f);
-  out->col.insert(out->col.end(), 4, 0u);
+  out->val.insert(out->val.end(), 32 * kQuadBundle, 0.f);
+  out->col.insert(out->col.end(), 4 * kQuadBundle, 0u);
   return true;
 }
 
@@ -492,11 +512,17 @@ bool validate_quad(const HostQuad& h, std::string* err) {
       if (r[3] < 0 || r[7] < 1 || r[7] > kQuadTile || r[3] + r[7] > nr) return bad("tile rows");
       for (int pass = 0; pass < 2; ++pass) {
         const int v = r[4 * pass], c = r[4 * pass + 1], n = r[4 * pass + 2], unit = pass == 0 ? 2 : 4;
-        if (n < 0 || n % unit || v < 0 || v % 8 || c < 0 || c % 4) return bad("tile alignment");
-        if ((size_t)4 * v + (size_t)n * 32 / unit + 32 > h.val.size() || (size_t)c + n + 4 > h.col.size())
+        if (n < 0 || n % unit || v < 0 || c < 0 || c % unit) return bad("tile alignment");
+        // the last read is the step past the end
+        const size_t steps = n / unit;
+        if (4 * (v + (steps * 8 + 7) * kQuadBundle + 1) > h.val.size() ||
+            c + steps * kQuadBundle * unit + unit > h.col.size())
           return bad("tile extent");
-        for (int k = c; k < c + n; ++k)
-          if (h.col[k] % step || (int)(h.col[k] / step) >= nr) return bad("tile column");
+        for (size_t k = 0; k < steps; ++k)
+          for (int u = 0; u < unit; ++u) {
+            const uint32_t o = h.col[c + k * kQuadBundle * unit + u];
+            if (o % step || (int)(o / step) >= nr) return bad("tile column");
+          }
       }
     }
   }
