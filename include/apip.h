@@ -329,7 +329,8 @@ apip_status apip_check_bounds_selftest(apip_ctx* ctx, void* stream);
  *   [4] sum over the records of their segment length
  *   [5] pool: sum over the pool values of the length of their reverse row
  *   [6] pool: C -> A back-propagation entries
- *   [7] compacted atoms per ACE thread block
+ *   [7] compacted atoms per ACE thread block (streamed with ace_group 0: of a large
+ *       system; the kernel takes 2, 4, 8 or 32 by their number)
  *   [8] ACE thread blocks per launch
  *   [9] evaluation: 0 = pool, 1 = streamed
  *   [10] floating-point operations per compacted atom of the table work (forward

@@ -16,6 +16,8 @@
 // Steps 1 and 4 are those of ace_device.cuh.
 #pragma once
 
+#include <algorithm>
+
 #include "ace_device.cuh"
 #include "gaunt_layout.h"
 
@@ -204,17 +206,13 @@ __device__ __forceinline__ bool record_ok(int* status, const Rec<T>& rc, int nA)
 }
 #endif
 
+// The whole evaluation with NAT atoms per block, for all compacted atoms.
 template <typename T, typename K, int LMAX, int NAT>
-__global__ void __launch_bounds__(kAceThreads, 2) k_ace_stream(Args<T> a, AceDev<T> t) {
-  pdl_begin();
-  // every list-build kernel of this call has completed: block 0 clears the
-  // trigger (and, after a build, the binning counts) for the next step
-  if (blockIdx.x == 0) end_list_build(a.flags, a.cell_count, a.ncell);
+__device__ __forceinline__ void stream_body(const Args<T>& a, const AceDev<T>& t, unsigned char* smem_raw, void* group) {
   static_assert(NAT <= 32 && 32 % NAT == 0, "a warp holds whole slices");
   constexpr int NS = kAceThreads / NAT;
   constexpr bool PRIV = stream_private<T, LMAX>();
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ AceGroup<T, NAT> g;
+  AceGroup<T, NAT>& g = *static_cast<AceGroup<T, NAT>*>(group);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int ka = tid % NAT, slice = tid / NAT;
   const int nA = t.nA;
@@ -371,51 +369,77 @@ __global__ void __launch_bounds__(kAceThreads, 2) k_ace_stream(Args<T> a, AceDev
   block_energy<T, NAT>(a, g, e_part);
 }
 
-template <typename T, typename K, int LMAX, int NAT>
-void launch_stream_lk(const Args<T>& a, const AceDev<T>& t, int blocks, cudaStream_t s) {
-  const size_t bytes = ace_stream_smem<T, LMAX, NAT>(t.nA);
-  cudaFuncSetAttribute(k_ace_stream<T, K, LMAX, NAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  launch_pdl(k_ace_stream<T, K, LMAX, NAT>, blocks, kAceThreads, bytes, s, a, t);
+// Atoms per block (t.group, or by the number of compacted atoms where it is 0).  A
+// block's time is a serial chain over its slices' couplings, shorter with fewer atoms
+// (hence more slices): float32 about 30, 38, 47 and 105 us for 2, 4, 8 and 32, but the
+// table reads and the sums over the slices are per block, so that large counts want
+// large groups.  So: 2 while each SM has at most one block, 4 for one round of the
+// resident blocks, 8 for two rounds, 32 beyond (measured for every group at 100 to
+// 79 k compacted atoms in both precisions; whole call at 2000, 1 % of them
+// compacted: 65 -> 48 us, in float64 481 -> 295 us; all of them, 8 instead of 32:
+// 125 -> 65 us and 1069 -> 787 us).
+template <typename T, typename K, int LMAX>
+__global__ void __launch_bounds__(kAceThreads, 2) k_ace_stream(Args<T> a, AceDev<T> t) {
+  pdl_begin();
+  // every list-build kernel of this call has completed: block 0 clears the
+  // trigger (and, after a build, the binning counts) for the next step
+  if (blockIdx.x == 0) end_list_build(a.flags, a.cell_count, a.ncell);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ __align__(16) unsigned char group[sizeof(AceGroup<T, 32>)];
+  int nat = t.group;
+  if (nat == 0) {
+    const int count = a.counts[0], r = (int)gridDim.x;
+    nat = count <= 2 * t.sms ? 2 : count <= 4 * r ? 4 : count <= 16 * r ? 8 : 32;
+  }
+  switch (nat) {
+    case 2: stream_body<T, K, LMAX, 2>(a, t, smem_raw, group); break;
+    case 4: stream_body<T, K, LMAX, 4>(a, t, smem_raw, group); break;
+    case 8: stream_body<T, K, LMAX, 8>(a, t, smem_raw, group); break;
+    default: stream_body<T, K, LMAX, 32>(a, t, smem_raw, group); break;
+  }
 }
 
-template <typename T, typename K, int LMAX, int NAT>
+template <typename T, int LMAX>
+size_t stream_smem_max(int nA) {
+  return std::max(std::max(ace_stream_smem<T, LMAX, 2>(nA), ace_stream_smem<T, LMAX, 4>(nA)),
+                  std::max(ace_stream_smem<T, LMAX, 8>(nA), ace_stream_smem<T, LMAX, 32>(nA)));
+}
+
+template <typename T, typename K, int LMAX>
+void launch_stream_lk(const Args<T>& a, const AceDev<T>& t, int blocks, cudaStream_t s) {
+  const size_t bytes = stream_smem_max<T, LMAX>(t.nA);
+  cudaFuncSetAttribute(k_ace_stream<T, K, LMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  launch_pdl(k_ace_stream<T, K, LMAX>, blocks, kAceThreads, bytes, s, a, t);
+}
+
+template <typename T, typename K, int LMAX>
 int occupancy_stream_lk(int nA) {
-  const size_t bytes = ace_stream_smem<T, LMAX, NAT>(nA);
+  const size_t bytes = stream_smem_max<T, LMAX>(nA);
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (bytes + (size_t)1024 > (size_t)optin) return 0;
-  if (cudaFuncSetAttribute(k_ace_stream<T, K, LMAX, NAT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if (bytes + (size_t)2048 > (size_t)optin) return 0;
+  if (cudaFuncSetAttribute(k_ace_stream<T, K, LMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)bytes) != cudaSuccess)
     return 0;
   int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_ace_stream<T, K, LMAX, NAT>, kAceThreads, bytes) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_ace_stream<T, K, LMAX>, kAceThreads, bytes) !=
       cudaSuccess)
     return 0;
   return occ;
 }
 
-template <typename T, typename K, int NAT>
-int stream_k(const Args<T>* a, const AceDev<T>& t, int blocks, cudaStream_t s, bool query) {
+template <typename T, typename K>
+int stream_dispatch(const Args<T>* a, const AceDev<T>& t, int blocks, cudaStream_t s, bool query) {
   switch (t.l_max) {
 #define APIP_CASE(L)                                           \
   case L:                                                      \
-    if (query) return occupancy_stream_lk<T, K, L, NAT>(t.nA); \
-    launch_stream_lk<T, K, L, NAT>(*a, t, blocks, s);          \
+    if (query) return occupancy_stream_lk<T, K, L>(t.nA);      \
+    launch_stream_lk<T, K, L>(*a, t, blocks, s);               \
     return 0;
     APIP_CASE(0) APIP_CASE(1) APIP_CASE(2) APIP_CASE(3)
     default: APIP_CASE(4)
 #undef APIP_CASE
-  }
-}
-
-template <typename T, typename K>
-int stream_dispatch(const Args<T>* a, const AceDev<T>& t, int blocks, cudaStream_t s, bool query) {
-  switch (t.group) {
-    case 32: return stream_k<T, K, 32>(a, t, blocks, s, query);
-    case 8: return stream_k<T, K, 8>(a, t, blocks, s, query);
-    case 4: return stream_k<T, K, 4>(a, t, blocks, s, query);
-    default: return 0;
   }
 }
 

@@ -331,6 +331,7 @@ AceDev<T> ace_dev(apip_ctx* c) {
   t.two_over_rc = T(2.0 / p.ace_rc);
   t.inv_width = T(1.0 / p.ace_rc_width);
   t.kind = c->ace_kind;
+  t.sms = c->sms;
   t.nC = c->ace_nC;
   t.npool = c->ace_npool;
   unsigned char* b = static_cast<unsigned char*>(c->ace_tab);
@@ -585,11 +586,8 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->dev);
   ctx->sms = std::max(1, sms);
   // atoms per ACE block.  Pool kernel: the largest group whose pools leave room
-  // for two resident blocks per SM, else the largest that fits.  Streamed
-  // kernel: 8 atoms per block for the adaptive switches (a few thousand
-  // compacted atoms fill the resident blocks in one round; 4 per block took two
-  // rounds and 28 % longer on the 249 k-atom void crystal), 32 for constant lam
-  // (every atom compacted).
+  // for two resident blocks per SM, else the largest that fits.  Streamed kernel:
+  // on the device, by the number of compacted atoms.
   {
     const bool f32 = p->precision == APIP_FP32;
     auto occ_of = [&](int g) {
@@ -608,15 +606,10 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
       t.l_max = p->ace_l_max; t.nA = nA; t.qrows = hq.rows;
       group = kQuadAtoms;
       occ = ace_quad_occupancy(t);
+    } else if (streamed) {
+      if (group == 0 || group == 4 || group == 8 || group == 32) occ = occ_of(group);
     } else if (group != 0) {
       occ = occ_of(group);   // 0 for a group the kernel does not provide
-    } else if (streamed) {
-      const bool adaptive = p->lam_mode == APIP_LAM_PAPER || p->lam_mode == APIP_LAM_LEARNED;
-      const int order_a[3] = {8, 4, 32}, order_c[3] = {32, 8, 4};
-      for (int q = 0; q < 3 && occ == 0; ++q) {
-        group = adaptive ? order_a[q] : order_c[q];
-        occ = occ_of(group);
-      }
     } else {
       for (int g : {8, 4, 2, 1}) {
         const int o = occ_of(g);
@@ -795,7 +788,9 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
     // rows 4 per element, C -> A entries 3 each
     info[10] = 3 * info[2] + 2 * info[4] + 4 * info[3] + 4 * info[5] + 3 * info[6];
   }
-  ctx->ace_info[7] = ctx->ace_group;
+  // (streamed without a group asked for: the group of a large system)
+  ctx->ace_info[7] = ctx->ace_group != 0 ? ctx->ace_group
+                     : p->lam_mode == APIP_LAM_PAPER || p->lam_mode == APIP_LAM_LEARNED ? 8 : 32;
   ctx->ace_info[8] = ctx->ace_blocks;
   ctx->ace_info[9] = streamed ? 1 : 0;
   APIP_ALLOC(ctx->ace_tab, host.size());

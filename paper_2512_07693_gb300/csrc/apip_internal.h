@@ -117,7 +117,8 @@ struct AceDev {
   const ulonglong2* qval;       // values
   const uint32_t* qcol;         // columns as offsets of their rows in X_L
   int qrows;                    // most values of X_L per atom
-  int group;                    // compacted atoms per thread block
+  int group;                    // compacted atoms per thread block (streamed: 0 = by their number, on the device)
+  int sms;                      // SMs of the device
 };
 
 struct HostStream {
@@ -241,7 +242,7 @@ struct apip_ctx {
   size_t ace_off[8] = {};
   int ace_qrows = 0;
   int ace_nf = 0, ace_npc = 0, ace_nC = 0, ace_npool = 0;
-  int ace_group = 1;
+  int ace_group = 1;           // (streamed: 0 = chosen on the device)
   int ace_kind = 0, ace_npr = 0, ace_ncpl = 0, ace_npart = 0;
   int64_t ace_info[APIP_ACE_INFO_COUNT] = {};
 
