@@ -63,15 +63,16 @@ __device__ __forceinline__ void features(T r, T fc, T dfc, T* phi, T* dphi) {
   }
 }
 
-// Descriptors of atom i over its neighbour list (r < rc of the ACE).
-template <typename T>
-__device__ __forceinline__ void descriptors_of(const Args<T>& a, int i, T* G) {
+// Descriptors of atom i over the entries g, g + LANES, ... of its neighbour list
+// (r < rc of the ACE).
+template <typename T, int LANES = 1>
+__device__ __forceinline__ void descriptors_of(const Args<T>& a, int i, T* G, int g = 0) {
 #pragma unroll
   for (int m = 0; m < kIn; ++m) G[m] = T(0);
   const auto si = a.pv.self(i);
   const T rc2 = a.ace_rc * a.ace_rc, inv_w = T(1) / (a.ace_rc - a.ace_rc_lo);
   const int cnt = APIP_CHK(a.status, BND_LIST_LEN, a.nnb[i], a.max_nb + 1);
-  for (int s = 0; s < cnt; ++s) {
+  for (int s = g; s < cnt; s += LANES) {
     const int j = APIP_CHK(a.status, BND_NEIGHBOUR, a.nbl[(size_t)s * a.nmax + i], a.n);
     const auto d = a.pv.vec(si, j);
     const T r2 = dot3(d, d);
@@ -244,7 +245,9 @@ __device__ __forceinline__ void split3(float x, float y, uint32_t& hi, uint32_t&
 // of the nearest one, |r - mu_m| < 8.5 dmu = 0.96 A; the others are below
 // exp(-eta (8.5 dmu)^2) = 1.3e-9 of the largest, under float32 rounding of the
 // sum.  Same ratio recurrence as features() outward from the nearest Gaussian.
+// STRIDE: distance of consecutive columns.
 constexpr int kWin = 8;
+template <int STRIDE = 1>
 __device__ __forceinline__ void add_features_window(float r, float fc, float kappa, float* row) {
   const float dmu = float(kDmu), eta = float(kEta);
   int m0 = __float2int_rn((r - float(kMu0)) / dmu);
@@ -253,15 +256,15 @@ __device__ __forceinline__ void add_features_window(float r, float fc, float kap
   const float base = -eta * dmu * dmu, slope = 2.f * eta * dmu * x0;
   const float e0 = __expf(-eta * x0 * x0) * fc;
   float rho = __expf(base + slope), sig = __expf(base - slope), up = e0, dn = e0;
-  row[m0] += e0;
+  row[m0 * STRIDE] += e0;
 #pragma unroll
   for (int k = 1; k <= kWin; ++k) {
     up *= rho;
     rho *= kappa;
     dn *= sig;
     sig *= kappa;
-    if (m0 + k < kIn) row[m0 + k] += up;
-    if (m0 - k >= 0) row[m0 - k] += dn;
+    if (m0 + k < kIn) row[(m0 + k) * STRIDE] += up;
+    if (m0 - k >= 0) row[(m0 - k) * STRIDE] += dn;
   }
 }
 
@@ -416,17 +419,20 @@ __device__ __forceinline__ float dfeatures_window(float r, float fc, float dfc, 
 
 // Pass 1 of the learned switch, float32, CUDA-core part: one thread per atom
 // walks its list for the EAM density, energy and xi' (as k_pass1) and the radial
-// descriptors, accumulated in the thread's shared-memory row (odd stride: the
-// lanes add at nearby Gaussian indices in different banks), and writes
-// x0 = G / 4 (float32, 32 per atom) for the network (k_learned_tc<false>).
+// descriptors, accumulated in the thread's shared-memory column [Gaussian][thread], and
+// writes x0 = G / 4 (float32, 32 per atom) for the network (k_learned_tc<false>).
+// Bound by issue: 17 of the 32 Gaussians, each a shared-memory read and write.  A
+// thread's column stays in its own bank whatever Gaussians the lanes are at; with a row
+// of 33 per thread the lanes met in three or four banks at a time, which bound the
+// kernel (900 k atoms: 544 us).
 __global__ void __launch_bounds__(kBlock) k_learned_desc(Args<float> a, float* __restrict__ x0) {
   pdl_begin();
-  __shared__ float rows[kBlock * (kIn + 1)];
+  __shared__ float rows[kBlock * kIn];
   __shared__ double sh[32];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  float* row = rows + threadIdx.x * (kIn + 1);
+  float* row = rows + threadIdx.x;
 #pragma unroll
-  for (int m = 0; m < kIn; ++m) row[m] = 0.f;
+  for (int m = 0; m < kIn; ++m) row[m * kBlock] = 0.f;
   double e_out = 0.0;
   if (i < a.n) {
     const auto si = a.pv.self(i);
@@ -449,7 +455,7 @@ __global__ void __launch_bounds__(kBlock) k_learned_desc(Args<float> a, float* _
                 if (r2 < rc2) {
                   float dfc;
                   const float fc = ftrans(r, a.ace_rc_lo, a.ace_rc, inv_w, &dfc);
-                  add_features_window(r, fc, kappa, row);
+                  add_features_window<kBlock>(r, fc, kappa, row);
                 }
               });
     const float zz = zeta.value();
@@ -464,7 +470,8 @@ __global__ void __launch_bounds__(kBlock) k_learned_desc(Args<float> a, float* _
     float4* xo = reinterpret_cast<float4*>(x0 + (size_t)i * kIn);
 #pragma unroll
     for (int m = 0; m < kIn / 4; ++m)
-      xo[m] = make_float4(kSin * row[4 * m], kSin * row[4 * m + 1], kSin * row[4 * m + 2], kSin * row[4 * m + 3]);
+      xo[m] = make_float4(kSin * row[4 * m * kBlock], kSin * row[(4 * m + 1) * kBlock], kSin * row[(4 * m + 2) * kBlock],
+                          kSin * row[(4 * m + 3) * kBlock]);
   }
   const double tot = block_sum(e_out, sh);
   if (threadIdx.x == 0) a.partials[blockIdx.x] = tot;
@@ -798,14 +805,27 @@ __global__ void __launch_bounds__(128) k_mlp_force(Args<T> a) {
     mlp_force_atom(a, APIP_CHK(a.status, BND_COMPACT, a.clist[q], a.n));
 }
 
-template <typename T>
+// LANES threads per atom as in the passes (atom_lanes): at 2 k atoms one thread's chain
+// of some 60 entries, 32 Gaussians each, was the kernel's whole time (51 us).
+template <typename T, int LANES>
 __global__ void k_descriptors(Args<T> a, __nv_bfloat16* out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= a.n) return;
+  const int k = blockIdx.x * blockDim.x + threadIdx.x, i = k / LANES, g = k % LANES;
+  constexpr int MINE = kIn / LANES;
   T G[kIn];
-  descriptors_of(a, i, G);
+  if (i < a.n) {
+    descriptors_of<T, LANES>(a, i, G, g);
+  } else {
 #pragma unroll
-  for (int m = 0; m < kIn; ++m) out[(size_t)i * kIn + m] = __float2bfloat16_rn((float)G[m]);
+    for (int m = 0; m < kIn; ++m) G[m] = T(0);
+  }
+#pragma unroll
+  for (int o = 1; o < LANES; o <<= 1)
+#pragma unroll
+    for (int m = 0; m < kIn; ++m) G[m] += __shfl_xor_sync(0xffffffffu, G[m], o);
+  if (i >= a.n) return;
+#pragma unroll
+  for (int m = 0; m < kIn; ++m)
+    if (m / MINE == g) out[(size_t)i * kIn + m] = __float2bfloat16_rn((float)G[m]);
 }
 
 template <typename T>
@@ -893,7 +913,11 @@ template <typename T> void launch_mlp_force(const Args<T>& a, cudaStream_t s) {
 }
 
 template <typename T> void launch_descriptors(const Args<T>& a, uint16_t* out, cudaStream_t s) {
-  k_descriptors<T><<<(a.n + 127) / 128, 128, 0, s>>>(a, reinterpret_cast<__nv_bfloat16*>(out));
+  __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(out);
+  const int blocks = (int)(((int64_t)a.n * a.lanes + 127) / 128);
+  if (a.lanes == 8) k_descriptors<T, 8><<<blocks, 128, 0, s>>>(a, o);
+  else if (a.lanes == 4) k_descriptors<T, 4><<<blocks, 128, 0, s>>>(a, o);
+  else k_descriptors<T, 1><<<blocks, 128, 0, s>>>(a, o);
 }
 
 template <typename T> void launch_cast_params(const float* src, T* dst, cudaStream_t s) {
