@@ -13,15 +13,17 @@
 //  4. pair forces (ace_device.cuh).
 // No atomics, so the sums have a fixed order.
 //
-// What bounds it: float32 multiply-adds of the matrix products, 3.9 M per atom for
-// n_max 8, l_max 4 (2.95 M of them on entries that are not zero).  The record-wise pool kernel
-// (ace_pool.cuh) reads its 16-byte records, 5 MB forward and 20 MB back, once per
-// group of 1 to 4 atoms through L2; here 2.3 MB of values serve 8 atoms, and a
-// thread's tile of 8 rows by 4 values of X (one 16-byte read) has 64 accumulators, so
-// that 32 packed multiply-adds go with 4 uniform 16-byte loads and one of shared
-// memory.  8 atoms are what X_L and dE/dX_L of the largest degree leave room for
-// (2 x 89 KB); step 2 before step 3 instead of both channels' dE/dX_L kept apart
-// costs a fifth more multiply-adds and saves twice that space.
+// What bounds it: the loads of the matrix products.  They take 3.45 M multiply-adds per
+// atom for n_max 8, l_max 4 (2.95 M on entries that are not zero).  The record-wise pool
+// kernel (ace_pool.cuh) reads its 16-byte records, 5 MB forward and 20 MB back, once
+// per group of 1 to 4 atoms through L2; here 2.1 MB of values serve 8 atoms.  A thread's
+// tile is 4 rows (both channels) by the 8 atoms of one M: 32 packed multiply-adds for
+// two uniform 16-byte loads of values and two of X from shared memory (8 rows by 4
+// atoms: four and one, and every load of 16 bytes a lane takes four cycles or more of
+// the load pipe however few addresses it has).  8 atoms are what X_L and dE/dX_L of
+// the largest degree leave room for (2 x 89 KB); step 2 before step 3 instead of both
+// channels' dE/dX_L kept apart costs a fifth more multiply-adds and saves twice that
+// space.  Prefetching the values into L1 one to six steps ahead changed nothing.
 #pragma once
 
 #include "ace_device.cuh"
@@ -36,6 +38,13 @@ template <int LMAX>
 __host__ __device__ inline size_t ace_quad_smem(int nA, int rows) {
   const int xy = 2 * rows * kQuadAtoms, ry = (ry_elems<LMAX, kQuadThreads>() + 3) / 4 * 4;
   return sizeof(float) * (size_t)((xy > ry ? xy : ry) + 2 * nA * kQuadAtoms + kQuadThreads / 32 * kQuadAtoms);
+}
+
+// X_L and dE/dX_L: value M (of NM) of a row for atom k.  Four atoms lie together, so that
+// the lanes of a warp, on consecutive M, read consecutive 16 bytes.
+template <int NM>
+__device__ __forceinline__ int quad_at(int row, int M, int k) {
+  return (row * 2 + (k >> 2)) * (NM * 4) + M * 4 + (k & 3);
 }
 
 // Rows C_{(n1 L1)(n2 L2) LL} of X: four (n1, n2) and the 8 atoms per warp, chunk by chunk.
@@ -68,7 +77,7 @@ __device__ __forceinline__ void quad_form(const float* A, float* X, const short*
         }
       }
 #pragma unroll
-  for (int M = 0; M < NM; ++M) X[(row * NM + M) * kQuadAtoms + k] = C[M];
+  for (int M = 0; M < NM; ++M) X[quad_at<NM>(row, M, k)] = C[M];
 }
 
 // The part of dE/dA_{(n l)} (l = LT) that comes through its couplings of degree LL with
@@ -89,7 +98,7 @@ __device__ __forceinline__ void quad_back(const float* A, const float* Y, const 
 #pragma unroll
     for (int j = 0; j < NO; ++j) x[j] = two * A[(o * nlm + LO * LO + j) * kQuadAtoms + k];
 #pragma unroll
-    for (int M = 0; M < NM; ++M) y[M] = Y[(row * NM + M) * kQuadAtoms + k];
+    for (int M = 0; M < NM; ++M) y[M] = Y[quad_at<NM>(row, M, k)];
     int e = G0;
 #pragma unroll
     for (int i1 = 0; i1 < 2 * L1 + 1; ++i1)
@@ -107,18 +116,19 @@ __device__ __forceinline__ void quad_back(const float* A, const float* Y, const 
   }
 }
 
-// acc[r][j] += value(r) . X(column, j) over the columns of a tile; F2 rows are the two
-// channels of one row of S (NP = 8) or two rows of K2 (NP = 4).  The values of the
-// next step (2 or 4 columns) and their columns are loaded while these are used.
+// acc[r][j] += value(r) . X(column, atom j) over the columns of a tile; F2 rows are the
+// two channels of one row of S (NP = 4) or two rows of K2 (NP = 2).  Xq: the thread's M
+// in the first row, its last four atoms half further.  The values of the next step (2
+// or 4 columns) and their columns are loaded while these are used.
 template <int NP>
-__device__ __forceinline__ void quad_tile(const ulonglong2* val, const uint32_t* col, int len, const float* Xq,
-                                          F2 (&acc)[NP][4]) {
-  constexpr int U = 16 / NP;   // columns per step (128 bytes of values)
-  ulonglong2 vn[8];
+__device__ __forceinline__ void quad_tile(const ulonglong2* val, const uint32_t* col, int len, const float* Xq, int half,
+                                          F2 (&acc)[NP][kQuadAtoms]) {
+  constexpr int U = 8 / NP;   // columns per step (64 bytes of values)
+  ulonglong2 vn[4];
   uint32_t cn[U];
   auto fetch = [&](int st) {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) vn[q] = __ldg(val + (size_t)(st * 8 + q) * kQuadBundle);
+    for (int q = 0; q < 4; ++q) vn[q] = __ldg(val + (size_t)(st * 4 + q) * kQuadBundle);
     if constexpr (U == 2) {
       const uint2 c = __ldg(reinterpret_cast<const uint2*>(col + (size_t)st * kQuadBundle * U));
       cn[0] = c.x; cn[1] = c.y;
@@ -130,23 +140,23 @@ __device__ __forceinline__ void quad_tile(const ulonglong2* val, const uint32_t*
   fetch(0);
 #pragma unroll 1
   for (int st = 0; st < len / U; ++st) {
-    ulonglong2 v[8];
+    ulonglong2 v[4];
     uint32_t c[U];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = vn[q];
+    for (int q = 0; q < 4; ++q) v[q] = vn[q];
 #pragma unroll
     for (int u = 0; u < U; ++u) c[u] = cn[u];
     fetch(st + 1);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const float4 x = *reinterpret_cast<const float4*>(Xq + c[u]);
-      const F2 xd[4] = {f2(x.x), f2(x.y), f2(x.z), f2(x.w)};
+      const float4 x = *reinterpret_cast<const float4*>(Xq + c[u]), y = *reinterpret_cast<const float4*>(Xq + c[u] + half);
+      const F2 xd[kQuadAtoms] = {f2(x.x), f2(x.y), f2(x.z), f2(x.w), f2(y.x), f2(y.y), f2(y.z), f2(y.w)};
 #pragma unroll
       for (int r = 0; r < NP; ++r) {
         const ulonglong2 w = v[(u * NP + r) / 2];
         const F2 a{(r & 1) ? w.y : w.x};
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[r][j] = fma2(a, xd[j], acc[r][j]);
+        for (int j = 0; j < kQuadAtoms; ++j) acc[r][j] = fma2(a, xd[j], acc[r][j]);
       }
     }
   }
@@ -180,8 +190,8 @@ __device__ __forceinline__ void quad_rows(const AceDev<float>& t, int L, const f
   const int4 h = __ldg(t.qhdr + L);
   const int len = (2 * L + 1) * kQuadAtoms;
   for (int q = threadIdx.x; q < h.y * len; q += kQuadThreads) {
-    const int n = q / len;
-    X[h.x * len + q] = A[(n * NLM + L * L) * kQuadAtoms + q - n * len];
+    const int n = q / len, M = (q - n * len) / kQuadAtoms, k = q % kQuadAtoms;
+    X[((h.x + n) * 2 + (k >> 2)) * (len / 2) + M * 4 + (k & 3)] = A[(n * NLM + L * L + M) * kQuadAtoms + k];
   }
   if (L == 0 && threadIdx.x < kQuadAtoms) X[(h.x + h.y) * kQuadAtoms + threadIdx.x] = 1.f;
 }
@@ -223,7 +233,7 @@ __device__ __forceinline__ void quad_onto_a(const AceDev<float>& t, int L, const
 #pragma unroll
       for (int i = 0; i < 2 * LT + 1; ++i) {
         float v = W[(n * NLM + LT * LT + i) * kQuadAtoms + k] + g[i];
-        if (direct) v += Y[((h.x + n) * (2 * LT + 1) + i) * kQuadAtoms + k];
+        if (direct) v += Y[quad_at<2 * LT + 1>(h.x + n, i, k)];
         W[(n * NLM + LT * LT + i) * kQuadAtoms + k] = v;
       }
     };
@@ -235,16 +245,13 @@ __device__ __forceinline__ void quad_onto_a(const AceDev<float>& t, int L, const
   }
 }
 
-// Sums of f over the block per atom: thread parity tells which four atoms a thread has.
-// The totals are in red[0 .. 7] after the barrier.
-__device__ __forceinline__ void quad_sum(const Acc<float> (&f)[4], float* red) {
+// Sums of f over the block per atom, in red[0 .. 7] after the barrier.
+__device__ __forceinline__ void quad_sum(const Acc<float> (&f)[kQuadAtoms], float* red) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    float v = f[j].value();
-#pragma unroll
-    for (int o = 2; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane < 2) red[warp * kQuadAtoms + 4 * lane + j] = v;
+  for (int j = 0; j < kQuadAtoms; ++j) {
+    const float v = warp_sum(f[j].value());
+    if (lane == 0) red[warp * kQuadAtoms + j] = v;
   }
   __syncthreads();
   float s = 0.f;
@@ -272,7 +279,6 @@ __global__ void __launch_bounds__(kQuadThreads, 1) k_ace_quad(Args<float> a, Ace
   float* Y = X + t.qrows * NAT;
   const int count = a.counts[0];
   const int ngroups = (count + NAT - 1) / NAT;
-  const int half = tid & 1;                        // a thread's quads all hold these four atoms
   double e_part = 0.0;
 
   for (int grp = blockIdx.x; grp < ngroups; grp += gridDim.x) {
@@ -284,38 +290,38 @@ __global__ void __launch_bounds__(kQuadThreads, 1) k_ace_quad(Args<float> a, Ace
 
     // 2. phi_2 and F'(phi_2)
     {
-      Acc<float> f[4];
+      Acc<float> f[NAT];
       for (int L = 0; L <= 2 * LMAX; ++L) {
         const int4 h = __ldg(t.qhdr + L);
         quad_rows<K, LMAX>(t, L, A, X);
         __syncthreads();
-        const int nq = 2 * (2 * L + 1), step = 4 * nq;
-        for (int it = tid; it < h.w * nq; it += NT) {
-          const int tl = it / nq, q = it - tl * nq;
+        const int nm = 2 * L + 1, half = 4 * nm;
+        for (int it = tid; it < h.w * nm; it += NT) {
+          const int tl = it / nm, M = it - tl * nm;
           const int4 rb = __ldg(t.qtile + 2 * (h.z + tl)), ra = __ldg(t.qtile + 2 * (h.z + tl) + 1);
-          F2 acc[4][4];
+          if (ra.z == 0) continue;
+          F2 acc[2][NAT];
 #pragma unroll
-          for (int r = 0; r < 4; ++r)
+          for (int r = 0; r < 2; ++r)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc[r][j] = f2(0.f);
-          if (ra.z > 0) {
-            quad_tile<4>(t.qval + ra.x, t.qcol + ra.y, ra.z, X + 4 * q, acc);
-            float s[4] = {0.f, 0.f, 0.f, 0.f};
+            for (int j = 0; j < NAT; ++j) acc[r][j] = f2(0.f);
+          quad_tile<2>(t.qval + ra.x, t.qcol + ra.y, ra.z, X + 4 * M, half, acc);
+          float s[NAT] = {};
 #pragma unroll
-            for (int r = 0; r < kQuadTile; ++r) {
-              if (r < ra.w) {
-                const float4 x = *reinterpret_cast<const float4*>(X + (rb.w + r) * step + 4 * q);
-                const float xv[4] = {x.x, x.y, x.z, x.w};
+          for (int r = 0; r < kQuadTile; ++r) {
+            if (r < ra.w) {
+              const float* xp = X + (rb.w + r) * 2 * half + 4 * M;
+              const float4 x = *reinterpret_cast<const float4*>(xp), y = *reinterpret_cast<const float4*>(xp + half);
+              const float xv[NAT] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                  const float2 z = f2_get(acc[r / 2][j]);
-                  s[j] += xv[j] * ((r & 1) ? z.y : z.x);
-                }
+              for (int j = 0; j < NAT; ++j) {
+                const float2 z = f2_get(acc[r / 2][j]);
+                s[j] += xv[j] * ((r & 1) ? z.y : z.x);
               }
             }
-#pragma unroll
-            for (int j = 0; j < 4; ++j) f[j].add(s[j]);
           }
+#pragma unroll
+          for (int j = 0; j < NAT; ++j) f[j].add(s[j]);
         }
         __syncthreads();
       }
@@ -330,44 +336,44 @@ __global__ void __launch_bounds__(kQuadThreads, 1) k_ace_quad(Args<float> a, Ace
 
     // 3. phi_1 and the adjoint
     {
-      Acc<float> f[4];
-      float dfs[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) dfs[j] = g.dfs[4 * half + j];
+      Acc<float> f[NAT];
       for (int L = 0; L <= 2 * LMAX; ++L) {
         const int4 h = __ldg(t.qhdr + L);
         quad_rows<K, LMAX>(t, L, A, X);   // (dE/dX of the degree before is read only from Y)
         __syncthreads();
-        const int nq = 2 * (2 * L + 1), step = 4 * nq;
-        for (int it = tid; it < h.w * nq; it += NT) {
-          const int tl = it / nq, q = it - tl * nq;
+        const int nm = 2 * L + 1, half = 4 * nm;
+        for (int it = tid; it < h.w * nm; it += NT) {
+          const int tl = it / nm, M = it - tl * nm;
           const int4 rb = __ldg(t.qtile + 2 * (h.z + tl));
           const int nr = __ldg(reinterpret_cast<const int*>(t.qtile + 2 * (h.z + tl) + 1) + 3);
-          F2 acc[8][4];
+          F2 acc[kQuadTile][NAT];
 #pragma unroll
-          for (int r = 0; r < 8; ++r)
+          for (int r = 0; r < kQuadTile; ++r)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc[r][j] = f2(0.f);
-          quad_tile<8>(t.qval + rb.x, t.qcol + rb.y, rb.z, X + 4 * q, acc);
-          float s[4] = {0.f, 0.f, 0.f, 0.f};
+            for (int j = 0; j < NAT; ++j) acc[r][j] = f2(0.f);
+          quad_tile<kQuadTile>(t.qval + rb.x, t.qcol + rb.y, rb.z, X + 4 * M, half, acc);
+          float s[NAT] = {};
 #pragma unroll
           for (int r = 0; r < kQuadTile; ++r) {
             if (r < nr) {
-              const int o = (rb.w + r) * step + 4 * q;
-              const float4 x = *reinterpret_cast<const float4*>(X + o);
-              const float xv[4] = {x.x, x.y, x.z, x.w};
-              float y[4];
+              const int o = (rb.w + r) * 2 * half + 4 * M;
 #pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                const float2 z = f2_get(acc[r][j]);
-                s[j] += xv[j] * z.x;
-                y[j] = z.x + dfs[j] * z.y;
+              for (int b = 0; b < 2; ++b) {
+                const float4 x = *reinterpret_cast<const float4*>(X + o + b * half);
+                const float xv[4] = {x.x, x.y, x.z, x.w};
+                float y[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                  const float2 z = f2_get(acc[r][4 * b + j]);
+                  s[4 * b + j] += xv[j] * z.x;
+                  y[j] = z.x + g.dfs[4 * b + j] * z.y;
+                }
+                *reinterpret_cast<float4*>(Y + o + b * half) = make_float4(y[0], y[1], y[2], y[3]);
               }
-              *reinterpret_cast<float4*>(Y + o) = make_float4(y[0], y[1], y[2], y[3]);
             }
           }
 #pragma unroll
-          for (int j = 0; j < 4; ++j) f[j].add(0.5f * s[j]);
+          for (int j = 0; j < NAT; ++j) f[j].add(0.5f * s[j]);
         }
         __syncthreads();
         quad_onto_a<K, LMAX>(t, L, A, Y, W);

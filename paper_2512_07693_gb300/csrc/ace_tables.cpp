@@ -369,8 +369,8 @@ void gaunt4_fill(double* out) {
 // coefficients of both channels symmetrically (a square twice), K2_L those of
 // channel 2 once.  The function order p <= q <= s <= u leaves two thirds of S_L
 // empty, so a tile of kQuadTile rows keeps only the columns that one of its rows
-// has; with the rows ordered by (n_q, p) the tiles of an 8 / 4 basis hold 1.33 times
-// the entries that are there (ordered by (p, q) 1.68 times).  Tiles are listed by
+// has; with the rows ordered by (n_q, p) the tiles of an 8 / 4 basis hold 1.17 times
+// the entries that are there (ordered by (p, q) 1.34 times).  Tiles are listed by
 // falling length; the values of kQuadBundle of them are interleaved 16 bytes at a time,
 // so that the lanes of a warp, which work on up to that many tiles, read one line.
 bool build_quad(int n_max, int l_max, const double* c1, const double* c2, int64_t n_basis, HostQuad* out,
@@ -441,7 +441,7 @@ bool build_quad(int n_max, int l_max, const double* c1, const double* c2, int64_
           }
           if (any) t.cols[pass].push_back(c);
         }
-        const size_t unit = pass == 0 ? 2 : 4;   // columns per 128 bytes of values
+        const size_t unit = pass == 0 ? 2 : 4;   // columns per 64 bytes of values
         while (t.cols[pass].size() % unit) t.cols[pass].push_back(-1);
       }
       tiles.push_back(t);
@@ -457,7 +457,7 @@ bool build_quad(int n_max, int l_max, const double* c1, const double* c2, int64_
         size_t len = 0;
         for (size_t k = 0; k < nb; ++k) len = std::max(len, tiles[b + k].cols[pass].size());
         const size_t v0 = out->val.size(), k0 = out->col.size();
-        out->val.resize(v0 + len / unit * 32 * kQuadBundle, 0.f);
+        out->val.resize(v0 + len / unit * 16 * kQuadBundle, 0.f);
         out->col.resize(k0 + len * kQuadBundle, 0u);
         for (size_t k = 0; k < nb; ++k) {
           const Tile& t = tiles[b + k];
@@ -472,8 +472,8 @@ bool build_quad(int n_max, int l_max, const double* c1, const double* c2, int64_
             for (int r = 0; r < t.rows; ++r) {
               const size_t e = (size_t)(t.row + r) * nr + c;
               for (int ch = 0; ch < (pass == 0 ? 2 : 1); ++ch) {
-                const size_t f = pass == 0 ? u * 16 + 2 * r + ch : u * 8 + r;   // of the 32 values of this tile and step
-                out->val[v0 + ((step_i * 8 + f / 4) * kQuadBundle + k) * 4 + f % 4] =
+                const size_t f = pass == 0 ? u * 8 + 2 * r + ch : u * 4 + r;   // of the 16 values of this tile and step
+                out->val[v0 + ((step_i * 4 + f / 4) * kQuadBundle + k) * 4 + f % 4] =
                     (float)(pass == 1 ? k2[e] : ch == 0 ? s1[e] : s2[e]);
               }
             }
@@ -491,7 +491,7 @@ bool build_quad(int n_max, int l_max, const double* c1, const double* c2, int64_
     out->rows = std::max(out->rows, nr * (2 * L + 1));
   }
   // the loops read one step past a tile's last
-  out->val.insert(out->val.end(), 32 * kQuadBundle, 0.f);
+  out->val.insert(out->val.end(), 16 * kQuadBundle, 0.f);
   out->col.insert(out->col.end(), 4 * kQuadBundle, 0u);
   return true;
 }
@@ -515,7 +515,7 @@ bool validate_quad(const HostQuad& h, std::string* err) {
         if (n < 0 || n % unit || v < 0 || c < 0 || c % unit) return bad("tile alignment");
         // the last read is the step past the end
         const size_t steps = n / unit;
-        if (4 * (v + (steps * 8 + 7) * kQuadBundle + 1) > h.val.size() ||
+        if (4 * (v + (steps * 4 + 3) * kQuadBundle + 1) > h.val.size() ||
             c + steps * kQuadBundle * unit + unit > h.col.size())
           return bad("tile extent");
         for (size_t k = 0; k < steps; ++k)

@@ -86,7 +86,7 @@ template <typename T> struct alignas(sizeof(T) == 4 ? 8 : 16) Ent { T v; uint32_
 constexpr int kAcePool = 0, kAceStreamed = 1, kAceQuad = 2;
 constexpr int kQuadAtoms = 8;       // atoms per block of the quadratic evaluation
 constexpr int kQuadThreads = 384;   // its threads per block
-constexpr int kQuadTile = 8;        // rows of S_L per tile
+constexpr int kQuadTile = 4;        // rows of S_L per tile
 constexpr int kQuadBundle = 8;      // tiles whose values are interleaved
 constexpr int kQuadLs = 2 * kLmaxCap + 1;                       // degrees L of a coupling
 constexpr int kQuadMap = (kLmaxCap + 1) * (kLmaxCap + 1) * kNmaxCap * kNmaxCap;   // rowmap entries per degree
