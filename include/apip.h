@@ -113,11 +113,11 @@ typedef struct apip_params {
      n_max in [1, 8], l_max in [0, 4], nu_max in [1, 4], n_max (l_max+1)^2 <= 254. */
   int32_t ace_n_max, ace_l_max, ace_nu_max;
   int32_t ace_group;         /* compacted atoms per ACE thread block, or 0 = automatic.
-                                Body order <= 3 (streamed): 4, 8 or 32 (automatic: 8 for the
-                                paper and learned switches, 32 for constant lam).  Body
-                                order 4 (pool): 1, 2, 4 or 8 (automatic: the largest whose
-                                two per-atom pools leave room for two resident blocks per
-                                SM).  A group the evaluation does not provide, or whose
+                                Body order <= 3 (streamed): 4, 8 or 32 (automatic: 2, 4, 8
+                                or 32 by the number of compacted atoms).  Body order 4
+                                (pool): 1, 2, 4 or 8 (automatic in float64: the largest
+                                whose two per-atom pools leave room for two resident blocks
+                                per SM; in float32 the quadratic evaluation, 8).  A group the evaluation does not provide, or whose
                                 shared memory does not fit, is rejected by apip_create
                                 (APIP_ERR_ARG). */
   double ace_rc, ace_rc_width, ace_eps, ace_a_scale;
@@ -320,7 +320,9 @@ apip_status apip_check_bounds_selftest(apip_ctx* ctx, void* stream);
  * (host call, no device work).  Body order <= 3 uses the streamed evaluation
  * (couplings C_{(p1 p2) L M} = sum G A_{p1} A_{p2} formed in registers and
  * contracted with their nu = 3 partners), body order 4 the coupling pool (all C
- * of an atom stored, every basis function a dot product of two pool segments).
+ * of an atom stored, every basis function a dot product of two pool segments; in
+ * float32 with ace_group 0 these products as quadratic forms shared by 8 atoms, for
+ * which the pool's counts are given).
  * out (host, APIP_ACE_INFO_COUNT entries):
  *   [0] values per atom in shared memory: 1 + n_max (l_max+1)^2 (+ pool couplings)
  *   [1] couplings (streamed) or coupling components (pool)

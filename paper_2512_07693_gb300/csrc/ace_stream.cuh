@@ -374,7 +374,8 @@ __device__ __forceinline__ void stream_body(const Args<T>& a, const AceDev<T>& t
 // (hence more slices): float32 about 30, 38, 47 and 105 us for 2, 4, 8 and 32, but the
 // table reads and the sums over the slices are per block, so that large counts want
 // large groups.  So: 2 while each SM has at most one block, 4 for one round of the
-// resident blocks, 8 for two rounds, 32 beyond (measured for every group at 100 to
+// resident blocks, 8 for two rounds, 32 beyond (with an adaptive switch only where
+// that leaves as many blocks resident: t.top) (measured for every group at 100 to
 // 79 k compacted atoms in both precisions; whole call at 2000, 1 % of them
 // compacted: 65 -> 48 us, in float64 481 -> 295 us; all of them, 8 instead of 32:
 // 125 -> 65 us and 1069 -> 787 us).
@@ -389,7 +390,7 @@ __global__ void __launch_bounds__(kAceThreads, 2) k_ace_stream(Args<T> a, AceDev
   int nat = t.group;
   if (nat == 0) {
     const int count = a.counts[0], r = (int)gridDim.x;
-    nat = count <= 2 * t.sms ? 2 : count <= 4 * r ? 4 : count <= 16 * r ? 8 : 32;
+    nat = count <= 2 * t.sms ? 2 : count <= 4 * r ? 4 : count <= 16 * r || t.top == 8 ? 8 : 32;
   }
   switch (nat) {
     case 2: stream_body<T, K, LMAX, 2>(a, t, smem_raw, group); break;
@@ -399,26 +400,31 @@ __global__ void __launch_bounds__(kAceThreads, 2) k_ace_stream(Args<T> a, AceDev
   }
 }
 
+// Shared memory of a launch: of the group asked for, else of the largest one the kernel
+// may choose (t.top).
 template <typename T, int LMAX>
-size_t stream_smem_max(int nA) {
-  return std::max(std::max(ace_stream_smem<T, LMAX, 2>(nA), ace_stream_smem<T, LMAX, 4>(nA)),
-                  std::max(ace_stream_smem<T, LMAX, 8>(nA), ace_stream_smem<T, LMAX, 32>(nA)));
+size_t stream_smem_of(const AceDev<T>& t) {
+  const size_t m4 = ace_stream_smem<T, LMAX, 4>(t.nA), m8 = ace_stream_smem<T, LMAX, 8>(t.nA);
+  const size_t m32 = ace_stream_smem<T, LMAX, 32>(t.nA);
+  if (t.group != 0) return t.group == 4 ? m4 : t.group == 8 ? m8 : m32;
+  const size_t few = std::max(ace_stream_smem<T, LMAX, 2>(t.nA), std::max(m4, m8));
+  return t.top == 8 ? few : std::max(few, m32);
 }
 
 template <typename T, typename K, int LMAX>
 void launch_stream_lk(const Args<T>& a, const AceDev<T>& t, int blocks, cudaStream_t s) {
-  const size_t bytes = stream_smem_max<T, LMAX>(t.nA);
+  const size_t bytes = stream_smem_of<T, LMAX>(t);
   cudaFuncSetAttribute(k_ace_stream<T, K, LMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   launch_pdl(k_ace_stream<T, K, LMAX>, blocks, kAceThreads, bytes, s, a, t);
 }
 
 template <typename T, typename K, int LMAX>
-int occupancy_stream_lk(int nA) {
-  const size_t bytes = stream_smem_max<T, LMAX>(nA);
+int occupancy_stream_lk(const AceDev<T>& t) {
+  const size_t bytes = stream_smem_of<T, LMAX>(t);
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (bytes + (size_t)2048 > (size_t)optin) return 0;
+  if (bytes + (size_t)1024 > (size_t)optin) return 0;
   if (cudaFuncSetAttribute(k_ace_stream<T, K, LMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)bytes) != cudaSuccess)
     return 0;
@@ -434,7 +440,7 @@ int stream_dispatch(const Args<T>* a, const AceDev<T>& t, int blocks, cudaStream
   switch (t.l_max) {
 #define APIP_CASE(L)                                           \
   case L:                                                      \
-    if (query) return occupancy_stream_lk<T, K, L>(t.nA);      \
+    if (query) return occupancy_stream_lk<T, K, L>(t);         \
     launch_stream_lk<T, K, L>(*a, t, blocks, s);               \
     return 0;
     APIP_CASE(0) APIP_CASE(1) APIP_CASE(2) APIP_CASE(3)

@@ -280,7 +280,10 @@ Args<T> make_args(apip_ctx* c, const double* pos, const int* id, int n, double* 
   a.det = c->det ? 1 : 0; a.blk_cnt = c->blk_cnt;
   a.partials = c->partials;
   // one energy partial per pass-1 block, ahead of the ACE blocks' partials
-  if (p.lam_mode != APIP_LAM_LEARNED) a.n_part_p1 = nblk((int64_t)n * a.lanes);
+  if (p.lam_mode != APIP_LAM_LEARNED) {
+    const int pt = pass_threads(sizeof(T), a.lanes);
+    a.n_part_p1 = (int)std::max<int64_t>(1, ((int64_t)n * a.lanes + pt - 1) / pt);
+  }
   else if (sizeof(T) == 4) a.n_part_p1 = nblk(n);   // the descriptor kernel's blocks
   else a.n_part_p1 = (int)std::max<int64_t>(1, (n + kLearnedBlock - 1) / kLearnedBlock);
   a.force = force;
@@ -332,6 +335,7 @@ AceDev<T> ace_dev(apip_ctx* c) {
   t.inv_width = T(1.0 / p.ace_rc_width);
   t.kind = c->ace_kind;
   t.sms = c->sms;
+  t.top = c->ace_top;
   t.nC = c->ace_nC;
   t.npool = c->ace_npool;
   unsigned char* b = static_cast<unsigned char*>(c->ace_tab);
@@ -593,11 +597,11 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
     auto occ_of = [&](int g) {
       if (f32) {
         AceDev<float> t{};
-        t.kind = ctx->ace_kind; t.l_max = p->ace_l_max; t.nA = nA; t.npool = tab.npool; t.group = g;
+        t.kind = ctx->ace_kind; t.l_max = p->ace_l_max; t.nA = nA; t.npool = tab.npool; t.group = g; t.top = ctx->ace_top;
         return streamed ? ace_stream_occupancy<float>(t) : ace_pool_occupancy<float>(t);
       }
       AceDev<double> t{};
-      t.kind = ctx->ace_kind; t.l_max = p->ace_l_max; t.nA = nA; t.npool = tab.npool; t.group = g;
+      t.kind = ctx->ace_kind; t.l_max = p->ace_l_max; t.nA = nA; t.npool = tab.npool; t.group = g; t.top = ctx->ace_top;
       return streamed ? ace_stream_occupancy<double>(t) : ace_pool_occupancy<double>(t);
     };
     int group = p->ace_group, occ = 0;
@@ -608,6 +612,13 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
       occ = ace_quad_occupancy(t);
     } else if (streamed) {
       if (group == 0 || group == 4 || group == 8 || group == 32) occ = occ_of(group);
+      if (group == 0) {   // 32 atoms per block cost a large float64 basis its second resident block
+        const bool adaptive = p->lam_mode == APIP_LAM_PAPER || p->lam_mode == APIP_LAM_LEARNED;
+        ctx->ace_top = 8;
+        const int occ8 = occ_of(group);
+        if (occ >= occ8 || (!adaptive && occ >= 1)) ctx->ace_top = 32;
+        else occ = occ8;
+      }
     } else if (group != 0) {
       occ = occ_of(group);   // 0 for a group the kernel does not provide
     } else {
@@ -826,6 +837,7 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
     e = p->precision == APIP_FP64 ? ace_pool_set_norms<double>(norms, nn) : ace_pool_set_norms<float>(norms, nn);
   }
   if (e != cudaSuccess) return fail_create(e);
+  if (p->precision == APIP_FP64 && (e = exp_table_set()) != cudaSuccess) return fail_create(e);
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail_create(e);
   *out = ctx;

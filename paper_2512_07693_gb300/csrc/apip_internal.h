@@ -118,6 +118,7 @@ struct AceDev {
   const uint32_t* qcol;         // columns as offsets of their rows in X_L
   int qrows;                    // most values of X_L per atom
   int group;                    // compacted atoms per thread block (streamed: 0 = by their number, on the device)
+  int top;                      // ... the largest of these, 8 or 32
   int sms;                      // SMs of the device
 };
 
@@ -243,6 +244,7 @@ struct apip_ctx {
   int ace_qrows = 0;
   int ace_nf = 0, ace_npc = 0, ace_nC = 0, ace_npool = 0;
   int ace_group = 1;           // (streamed: 0 = chosen on the device)
+  int ace_top = 32;            // ... up to this many
   int ace_kind = 0, ace_npr = 0, ace_ncpl = 0, ace_npart = 0;
   int64_t ace_info[APIP_ACE_INFO_COUNT] = {};
 

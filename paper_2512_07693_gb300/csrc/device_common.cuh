@@ -45,6 +45,17 @@ __device__ __forceinline__ T ftrans(T x, T lo, T hi, T inv_w, T* deriv) {
   return T(0.0625) * p * p * p * (T(8) + t * (T(-9) + T(3) * t));
 }
 
+// The same in float64 for lo <= x < hi, without the two comparisons (they go to the
+// float64 pipe) and with the constants folded: 8 operations, 11 with the derivative,
+// for 11 and 15.
+__device__ __forceinline__ double ftrans_in(double x, double lo, double hi, double inv_w, double* deriv) {
+  const double t = (hi + lo - 2.0 * x) * inv_w;
+  const double u = 1.0 - t * t;
+  *deriv = u * u * (0.9375 * (-2.0 * inv_w));
+  const double p = 1.0 + t;
+  return p * p * p * (0.5 + t * (-0.5625 + 0.1875 * t));
+}
+
 // 1 - f_trans(x, lo, hi) and d(1 - f_trans)/dx.
 template <typename T>
 __device__ __forceinline__ T ftrans_c(T x, T lo, T hi, T inv_w, T* deriv) {
@@ -63,6 +74,33 @@ __device__ __forceinline__ T ftrans_c(T x, T lo, T hi, T inv_w, T* deriv) {
 template <typename T> __device__ __forceinline__ T fexp(T x);
 template <> __device__ __forceinline__ float fexp<float>(float x) { return __expf(x); }
 template <> __device__ __forceinline__ double fexp<double>(double x) { return exp(x); }
+
+// exp(x) in float64 by Tang's table method (P. T. P. Tang, ACM Trans. Math. Softw. 15
+// (1989) 144): x = (256 k + j) ln2 / 256 + r, exp(x) = 2^k 2^(j/256) exp(r), |r| <=
+// ln2 / 512, the table holding 2^(j/256) as a sum of two doubles.  exp(r) - 1 = r +
+// r^2 (1/2 + r (c3 + r / 24)); c3 = 1/6 + 0.87 h^2 / 120, h = ln2 / 512, takes up the
+// quintic term (left: 5e-18).  Ten float64 operations, within 0.6 ulp; the library's
+// function takes some 25 on this GPU's slow float64 pipe.  Outside |x| < 690 (and for
+// a NaN) the library's.
+constexpr int kExpTab = 256;
+static __device__ __noinline__ double exp_far(double x) { return exp(x); }
+__device__ __forceinline__ double exp_tab(const double2* tab, double x) {
+  if ((unsigned)(__double2hiint(x) & 0x7fffffff) >= 0x40859000u) return exp_far(x);
+  constexpr double kLn2 = 0.69314718055994530942, kMagic = 6755399441055744.0;   // 1.5 2^52
+  constexpr double kStep = kLn2 / kExpTab;
+  constexpr double kHi = (double)(long long)(kStep * 281474976710656.0) / 281474976710656.0;   // 39 bits: k kHi is exact
+  constexpr double kLo = 2.8792978770186714e-15;   // ln2 / 256 - kHi
+  const double t = fma(x, kExpTab / kLn2, kMagic);
+  const int n = __double2loint(t);
+  const double k = t - kMagic;
+  const double r = fma(k, -kLo, fma(k, -kHi, x));
+  constexpr double h = kLn2 / (2 * kExpTab);
+  const double q = fma(r, fma(r, 1.0 / 24.0, 1.0 / 6.0 + 0.87 * h * h / 120.0), 0.5);
+  const double p = fma(r * r, q, r);
+  const double2 T = tab[n & (kExpTab - 1)];
+  const double v = T.x + fma(T.x, p, T.y);
+  return __hiloint2double(__double2hiint(v) + (n >> 8) * 1048576, __double2loint(v));
+}
 
 // Running sum with Kahan compensation in FP32; plain in FP64.
 template <typename T> struct Acc {

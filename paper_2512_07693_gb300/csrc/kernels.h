@@ -224,6 +224,14 @@ inline int atom_lanes(int64_t n, int sms) {
   return 8 * n <= fill ? 8 : (4 * n <= fill ? 4 : 1);
 }
 
+// Threads per block of pass 1 and pass 2.  In float64 with a thread per atom an SM's
+// pipe is the limit, and a few large blocks per SM leave it idle at the end (93 k atoms
+// in 363 blocks of 256: 65 % of the pipe for 86 % while blocks run).  With several
+// threads per atom blocks of 64 make the passes themselves faster at 2 k atoms (39 ->
+// 27 and 33 -> 24 us), but not the step, in which the kernels after them start early
+// (318 -> 410 us); in float32 they gain nothing (27 k atoms).
+inline int pass_threads(size_t elem, int lanes) { return elem == 8 && lanes == 1 ? 128 : kBlock; }
+
 // Launch with programmatic stream serialization (the kernel must start with
 // pdl_begin()).
 template <typename... KArgs, typename... Act>
@@ -250,6 +258,7 @@ template <typename T> void launch_prep(const Args<T>& a, cudaStream_t s);
 template <typename T> void launch_neighbors(const Args<T>& a, int ncell, cudaStream_t s);
 void launch_csp_init(const Args<double>& a, cudaStream_t s);
 void launch_set_csp(const int32_t* src, int* dst, int n, int nnb, cudaStream_t s);
+cudaError_t exp_table_set();   // float64 contexts: before the first pass 1
 template <typename T> void launch_pass1(const Args<T>& a, cudaStream_t s);
 template <typename T> void launch_pass2(const Args<T>& a, cudaStream_t s);
 // force mixing: append to the compacted list every atom with lam = 0 that has a

@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
+#include <vector>
 
 #include "kernels.h"
 #include "pair2.cuh"
@@ -681,8 +683,18 @@ __device__ __noinline__ EamTerm eam_rare(const PassK<float>& k, float r) {
 // The EAM sums read only the first nnb_e list entries (the pairs that can be
 // within the EAM cutoff).  FP32 path: also writes posg[i] = (posq[i], g_i) for
 // pass 2.
+// FP64 path: with one thread per atom bound by the float64 pipe, some 65 operations a
+// pair with exp_tab's table in shared memory (tab), 100 with the library's exponential
+// (249 k atoms, pass 1 and pass 2 with the shorter taper and smaller blocks: the step
+// 3.16 -> 2.81 ms).  A small system is not bound by it and loses more by the table's
+// loads and barrier in front of each short kernel (2 k atoms: 318 us a step without,
+// 355 with it).
+__device__ double2 g_exp_tab[kExpTab];
 template <typename T, int LANES>
-__device__ __forceinline__ void eam_sums(const Args<T>& a, int i, int g, T* zeta_out, T* pair_out) {
+__host__ __device__ constexpr bool exp_by_table() { return sizeof(T) == 8 && LANES == 1; }
+
+template <typename T, int LANES>
+__device__ __forceinline__ void eam_sums(const Args<T>& a, int i, int g, const double2* tab, T* zeta_out, T* pair_out) {
   const auto si = a.pv.self(i);
   const int end0 = APIP_CHK(a.status, BND_LIST_LEN, a.nnb_0[i], a.max_nb + 1);
   int end = APIP_CHK(a.status, BND_LIST_LEN, a.nnb_e[i], a.max_nb + 1);
@@ -737,9 +749,10 @@ __device__ __forceinline__ void eam_sums(const Args<T>& a, int i, int g, T* zeta
         T r, ir;
         len_inv(r2, &r, &ir);
         T fc = T(1), dfc = T(0);
-        if (!less_pos(r, rlo)) fc = ftrans(r, rlo, rc, inv_w, &dfc);
-        const T er = a.k.eam_A * fexp(-a.k.eam_beta * (r - a.k.eam_re));
-        const T x = fexp(-a.k.eam_alpha * (r - a.k.eam_r0));
+        if (!less_pos(r, rlo)) fc = ftrans_in(r, rlo, rc, inv_w, &dfc);
+        auto expo = [&](T v) { return exp_by_table<T, LANES>() ? exp_tab(tab, v) : fexp(v); };
+        const T er = a.k.eam_A * expo(-a.k.eam_beta * (r - a.k.eam_re));
+        const T x = expo(-a.k.eam_alpha * (r - a.k.eam_r0));
         const T q = x * x - T(2) * x;
         zeta += er * fc;
         pair += a.k.eam_D * q * fc;
@@ -862,6 +875,11 @@ template <typename T, int LANES>
 __global__ void __launch_bounds__(kBlock) k_pass1(Args<T> a) {
   pdl_begin();
   __shared__ double sh[32];
+  __shared__ double2 tab[exp_by_table<T, LANES>() ? kExpTab : 1];
+  if constexpr (exp_by_table<T, LANES>()) {
+    for (int k = threadIdx.x; k < kExpTab; k += blockDim.x) tab[k] = g_exp_tab[k];
+    __syncthreads();
+  }
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int g = LANES == 1 ? 0 : (int)(threadIdx.x % LANES);
   const bool active = t / LANES < a.n;
@@ -869,7 +887,7 @@ __global__ void __launch_bounds__(kBlock) k_pass1(Args<T> a) {
   if (LANES > 1 || active) {
     const int i = LANES == 1 ? t : min(t / LANES, a.n - 1);   // (LANES > 1: the warp stays whole for its shuffles)
     T z, pair;
-    eam_sums<T, LANES>(a, i, g, &z, &pair);
+    eam_sums<T, LANES>(a, i, g, tab, &z, &pair);
     const T gi = a.lam_mode == APIP_LAM_PAPER ? csp_g<T, LANES>(a, i, g) : T(0);
     if (active && g == 0) {
       const T sz = z > T(0) ? sqrt(z) : T(0);
@@ -1003,7 +1021,7 @@ __device__ __forceinline__ Pass2Sums<double> pass2_sums(const Args<double>& a, i
       } else {
         double r, ir, dw;
         len_inv(r2, &r, &ir);
-        const double w = ftrans(r, k.sw_r_w_lo, k.sw_r_w, k.sw_inv_w, &dw);
+        const double w = ftrans_in(r, k.sw_r_w_lo, k.sw_r_w, k.sw_inv_w, &dw);
         wbar += w;
         S += gj * w;
       }
@@ -1428,9 +1446,22 @@ void launch_csp_init(const Args<double>& a, cudaStream_t s) {
 }
 
 template <typename T> void launch_pass1(const Args<T>& a, cudaStream_t s) {
-  if (a.lanes == 8) launch_pdl(k_pass1<T, 8>, nblocks(8 * a.n), kBlock, 0, s, a);
-  else if (a.lanes == 4) launch_pdl(k_pass1<T, 4>, nblocks(4 * a.n), kBlock, 0, s, a);
-  else launch_pdl(k_pass1<T, 1>, nblocks(a.n), kBlock, 0, s, a);
+  const int pt = pass_threads(sizeof(T), a.lanes);
+  if (a.lanes == 8) launch_pdl(k_pass1<T, 8>, nblocks(8 * a.n, pt), pt, 0, s, a);
+  else if (a.lanes == 4) launch_pdl(k_pass1<T, 4>, nblocks(4 * a.n, pt), pt, 0, s, a);
+  else launch_pdl(k_pass1<T, 1>, nblocks(a.n, pt), pt, 0, s, a);
+}
+
+// The table of exp_tab on the current device: 2^(j / 256) rounded, and what that
+// leaves to 60 binary places.
+cudaError_t exp_table_set() {
+  std::vector<double2> h(kExpTab);
+  for (int j = 0; j < kExpTab; ++j) {
+    const long double v = exp2l((long double)j / kExpTab);
+    const double hi = (double)v;
+    h[j] = make_double2(hi, (double)(rintl((v - (long double)hi) * 0x1p60L) * 0x1p-60L));
+  }
+  return cudaMemcpyToSymbol(g_exp_tab, h.data(), sizeof(double2) * kExpTab);
 }
 
 // Force mixing: the precise model's forces on the atoms with lam > 0 need E^prec
@@ -1478,9 +1509,10 @@ template <typename T> void launch_pass2(const Args<T>& a, cudaStream_t s) {
   // (the deterministic mode's compaction counts per 256 atoms: one thread per atom)
   const int lanes = a.det ? 1 : a.lanes;
   const bool paper = a.lam_mode == APIP_LAM_PAPER || a.lam_mode == APIP_LAM_LEARNED;
-  if (lanes == 8) launch_pdl(paper ? k_pass2<T, true, 8> : k_pass2<T, false, 8>, nblocks(8 * a.n), kBlock, 0, s, a);
-  else if (lanes == 4) launch_pdl(paper ? k_pass2<T, true, 4> : k_pass2<T, false, 4>, nblocks(4 * a.n), kBlock, 0, s, a);
-  else launch_pdl(paper ? k_pass2<T, true, 1> : k_pass2<T, false, 1>, nblocks(a.n), kBlock, 0, s, a);
+  const int pt = pass_threads(sizeof(T), lanes);
+  if (lanes == 8) launch_pdl(paper ? k_pass2<T, true, 8> : k_pass2<T, false, 8>, nblocks(8 * a.n, pt), pt, 0, s, a);
+  else if (lanes == 4) launch_pdl(paper ? k_pass2<T, true, 4> : k_pass2<T, false, 4>, nblocks(4 * a.n, pt), pt, 0, s, a);
+  else launch_pdl(paper ? k_pass2<T, true, 1> : k_pass2<T, false, 1>, nblocks(a.n, pt), pt, 0, s, a);
   if (a.det) {
     launch_pdl(k_blk_scan, 1, 1024, 0, s, a.blk_cnt, nblocks(a.n));
     launch_pdl(k_compact_det<T>, nblocks(a.n), kBlock, 0, s, a);
