@@ -133,16 +133,30 @@ __device__ __forceinline__ bool less_pos(double x, double y) {
 }
 
 // r = |d| and 1/r from r^2: in float32 through the reciprocal square root
-// (rsqrtf, within 2 ulp); in float64 from the hardware's approximate reciprocal
-// square root y by Newton's iteration on both (each step an exact residual by a
-// multiply-add): ten float64 operations for the two, both within one ulp, where a
-// square root and a division take some twenty.
+// (rsqrtf, within 2 ulp; NaN and infinity for r^2 = 0); in float64 from the
+// hardware's approximate reciprocal square root y by Newton's iteration on both (each
+// step an exact residual by a multiply-add): ten float64 operations for the two, r
+// within one ulp and 1/r within two (a division by the rounded root is no better),
+// where a square root and a division take some twenty.  The iteration gives NaN for
+// zero (two atoms at one place: r = 0, 1/r = infinity, so that the pair's energy stays
+// finite), subnormal and infinite r^2: those, told by the exponent off the float64
+// pipe, go to the square root and the division.
 template <typename T> __device__ __forceinline__ void len_inv(T r2, T* r, T* ir);
 template <> __device__ __forceinline__ void len_inv<float>(float r2, float* r, float* ir) {
   *ir = rsqrtf(r2);
   *r = r2 * *ir;
 }
+static __device__ __noinline__ double2 len_inv_far(double r2) {
+  const double r = sqrt(r2);
+  return make_double2(r, 1.0 / r);
+}
 template <> __device__ __forceinline__ void len_inv<double>(double r2, double* r, double* ir) {
+  if ((unsigned)(__double2hiint(r2) - 0x00100000) >= 0x7fe00000u) {
+    const double2 v = len_inv_far(r2);
+    *r = v.x;
+    *ir = v.y;
+    return;
+  }
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r2));
   const double h = 0.5 * y;
