@@ -11,7 +11,15 @@
 //  3. for every L: X_L again, S_L^1 X_L and S_L^2 X_L in packed float pairs, phi_1,
 //     dE/dX_L, and that back onto A, each thread owning one segment A_{n l} of an atom;
 //  4. pair forces (ace_device.cuh).
-// No atomics, so the sums have a fixed order.
+// No atomics, so the sums have a fixed order.  The sum over a row's columns is plain, in
+// an order that puts the columns expected to be large last (build_quad); the rows'
+// contributions to phi are compensated per thread, and the block adds them up in
+// float-float.  In a restatement of the sums on the densities of cracked, void, vacancy
+// and bulk crystals (bases 4/4 to 8/4) the RMS error of phi against 64 bits is 0.42 to
+// 0.85 of the record-wise kernel's, which compensates per record; with the columns by
+// index and plain sums over rows and block it was 1.3 and 1.4 times as large (8/4, a
+// crack's faces).  Compensating within a row (every 16 or 32 columns) cost half and a
+// third more time for nothing beyond that.
 //
 // What bounds it: the loads of the matrix products.  They take 3.45 M multiply-adds per
 // atom for n_max 8, l_max 4 (2.95 M on entries that are not zero).  The record-wise pool
@@ -33,11 +41,11 @@
 namespace apip {
 
 // Dynamic shared memory: X_L and dE/dX_L (step 1 stages R, Y there), A, dE/dA and the
-// per-warp sums.
+// per-warp sums (high and low parts).
 template <int LMAX>
 __host__ __device__ inline size_t ace_quad_smem(int nA, int rows) {
   const int xy = 2 * rows * kQuadAtoms, ry = (ry_elems<LMAX, kQuadThreads>() + 3) / 4 * 4;
-  return sizeof(float) * (size_t)((xy > ry ? xy : ry) + 2 * nA * kQuadAtoms + kQuadThreads / 32 * kQuadAtoms);
+  return sizeof(float) * (size_t)((xy > ry ? xy : ry) + 2 * nA * kQuadAtoms + 2 * (kQuadThreads / 32) * kQuadAtoms);
 }
 
 // X_L and dE/dX_L: value M (of NM) of a row for atom k.  Four atoms lie together, so that
@@ -245,20 +253,29 @@ __device__ __forceinline__ void quad_onto_a(const AceDev<float>& t, int L, const
   }
 }
 
-// Sums of f over the block per atom, in red[0 .. 7] after the barrier.
-__device__ __forceinline__ void quad_sum(const Acc<float> (&f)[kQuadAtoms], float* red) {
+// Sums of f (pairs of atoms) over the block per atom, with what the compensated sums
+// still have to give back, in red[0 .. 7] after the barrier.
+__device__ __forceinline__ void quad_sum(const Acc2 (&f)[kQuadAtoms / 2], float* red) {
+  constexpr int NW = kQuadThreads / 32;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 #pragma unroll
   for (int j = 0; j < kQuadAtoms; ++j) {
-    const float v = warp_sum(f[j].value());
-    if (lane == 0) red[warp * kQuadAtoms + j] = v;
+    const float2 s = f2_get(f[j / 2].s), n = f2_get(f[j / 2].n);
+    FF v = (j & 1) ? FF{s.y, n.y} : FF{s.x, n.x};
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+      v = ff_add(v, FF{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)});
+    if (lane == 0) {
+      red[warp * kQuadAtoms + j] = v.hi;
+      red[(NW + warp) * kQuadAtoms + j] = v.lo;
+    }
   }
   __syncthreads();
-  float s = 0.f;
+  FF t{0.f, 0.f};
   if (tid < kQuadAtoms)
-    for (int w = 0; w < kQuadThreads / 32; ++w) s += red[w * kQuadAtoms + tid];
+    for (int w = 0; w < NW; ++w) t = ff_add(t, FF{red[w * kQuadAtoms + tid], red[(NW + w) * kQuadAtoms + tid]});
   __syncthreads();
-  if (tid < kQuadAtoms) red[tid] = s;
+  if (tid < kQuadAtoms) red[tid] = t.hi + t.lo;
   __syncthreads();
 }
 
@@ -275,7 +292,7 @@ __global__ void __launch_bounds__(kQuadThreads, 1) k_ace_quad(Args<float> a, Ace
   float* A = reinterpret_cast<float*>(smem_raw);   // A[c * 8 + k], then omega
   float* W = A + nA * NAT;                         // dE/dA
   float* red = W + nA * NAT;
-  float* X = red + NT / 32 * NAT;                  // X_L, then dE/dX_L (step 1 stages R, Y there)
+  float* X = red + 2 * (NT / 32) * NAT;                  // X_L, then dE/dX_L (step 1 stages R, Y there)
   float* Y = X + t.qrows * NAT;
   const int count = a.counts[0];
   const int ngroups = (count + NAT - 1) / NAT;
@@ -290,7 +307,7 @@ __global__ void __launch_bounds__(kQuadThreads, 1) k_ace_quad(Args<float> a, Ace
 
     // 2. phi_2 and F'(phi_2)
     {
-      Acc<float> f[NAT];
+      Acc2 f[NAT / 2];
       for (int L = 0; L <= 2 * LMAX; ++L) {
         const int4 h = __ldg(t.qhdr + L);
         quad_rows<K, LMAX>(t, L, A, X);
@@ -306,22 +323,24 @@ __global__ void __launch_bounds__(kQuadThreads, 1) k_ace_quad(Args<float> a, Ace
 #pragma unroll
             for (int j = 0; j < NAT; ++j) acc[r][j] = f2(0.f);
           quad_tile<2>(t.qval + ra.x, t.qcol + ra.y, ra.z, X + 4 * M, half, acc);
-          float s[NAT] = {};
 #pragma unroll
           for (int r = 0; r < kQuadTile; ++r) {
             if (r < ra.w) {
               const float* xp = X + (rb.w + r) * 2 * half + 4 * M;
-              const float4 x = *reinterpret_cast<const float4*>(xp), y = *reinterpret_cast<const float4*>(xp + half);
-              const float xv[NAT] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
 #pragma unroll
-              for (int j = 0; j < NAT; ++j) {
-                const float2 z = f2_get(acc[r / 2][j]);
-                s[j] += xv[j] * ((r & 1) ? z.y : z.x);
+              for (int b = 0; b < 2; ++b) {
+                const float4 x = *reinterpret_cast<const float4*>(xp + b * half);
+                float z[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                  const float2 u = f2_get(acc[r / 2][4 * b + j]);
+                  z[j] = (r & 1) ? u.y : u.x;
+                }
+                f[2 * b].add_prod(f2(x.x, x.y), f2(z[0], z[1]));
+                f[2 * b + 1].add_prod(f2(x.z, x.w), f2(z[2], z[3]));
               }
             }
           }
-#pragma unroll
-          for (int j = 0; j < NAT; ++j) f[j].add(s[j]);
         }
         __syncthreads();
       }
@@ -336,7 +355,7 @@ __global__ void __launch_bounds__(kQuadThreads, 1) k_ace_quad(Args<float> a, Ace
 
     // 3. phi_1 and the adjoint
     {
-      Acc<float> f[NAT];
+      Acc2 f[NAT / 2];   // of 2 phi_1
       for (int L = 0; L <= 2 * LMAX; ++L) {
         const int4 h = __ldg(t.qhdr + L);
         quad_rows<K, LMAX>(t, L, A, X);   // (dE/dX of the degree before is read only from Y)
@@ -352,7 +371,6 @@ __global__ void __launch_bounds__(kQuadThreads, 1) k_ace_quad(Args<float> a, Ace
 #pragma unroll
             for (int j = 0; j < NAT; ++j) acc[r][j] = f2(0.f);
           quad_tile<kQuadTile>(t.qval + rb.x, t.qcol + rb.y, rb.z, X + 4 * M, half, acc);
-          float s[NAT] = {};
 #pragma unroll
           for (int r = 0; r < kQuadTile; ++r) {
             if (r < nr) {
@@ -360,27 +378,26 @@ __global__ void __launch_bounds__(kQuadThreads, 1) k_ace_quad(Args<float> a, Ace
 #pragma unroll
               for (int b = 0; b < 2; ++b) {
                 const float4 x = *reinterpret_cast<const float4*>(X + o + b * half);
-                const float xv[4] = {x.x, x.y, x.z, x.w};
-                float y[4];
+                float z[4], y[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                  const float2 z = f2_get(acc[r][4 * b + j]);
-                  s[4 * b + j] += xv[j] * z.x;
-                  y[j] = z.x + g.dfs[4 * b + j] * z.y;
+                  const float2 u = f2_get(acc[r][4 * b + j]);
+                  z[j] = u.x;
+                  y[j] = u.x + g.dfs[4 * b + j] * u.y;
                 }
+                f[2 * b].add_prod(f2(x.x, x.y), f2(z[0], z[1]));
+                f[2 * b + 1].add_prod(f2(x.z, x.w), f2(z[2], z[3]));
                 *reinterpret_cast<float4*>(Y + o + b * half) = make_float4(y[0], y[1], y[2], y[3]);
               }
             }
           }
-#pragma unroll
-          for (int j = 0; j < NAT; ++j) f[j].add(0.5f * s[j]);
         }
         __syncthreads();
         quad_onto_a<K, LMAX>(t, L, A, Y, W);
       }
       quad_sum(f, red);
     }
-    if (tid < NAT) atom_scalars<float, NAT>(a, t, tid, red[tid], g.e[tid], g);
+    if (tid < NAT) atom_scalars<float, NAT>(a, t, tid, 0.5f * red[tid], g.e[tid], g);
     __syncthreads();
     for (int item = tid; item < nA * NAT; item += NT)
       W[item] *= t.a_scale * (a.force_mix ? 1.f : g.lam[item % NAT]);

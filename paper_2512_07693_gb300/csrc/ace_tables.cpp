@@ -370,7 +370,8 @@ void gaunt4_fill(double* out) {
 // channel 2 once.  The function order p <= q <= s <= u leaves two thirds of S_L
 // empty, so a tile of kQuadTile rows keeps only the columns that one of its rows
 // has; with the rows ordered by (n_q, p) the tiles of an 8 / 4 basis hold 1.17 times
-// the entries that are there (ordered by (p, q) 1.34 times).  Tiles are listed by
+// the entries that are there (ordered by (p, q) 1.34 times).  Its columns are ordered by
+// their expected size, for the rounding of their plain sum.  Tiles are listed by
 // falling length; the values of kQuadBundle of them are interleaved 16 bytes at a time,
 // so that the lanes of a warp, which work on up to that many tiles, read one line.
 bool build_quad(int n_max, int l_max, const double* c1, const double* c2, int64_t n_basis, HostQuad* out,
@@ -426,6 +427,17 @@ bool build_quad(int n_max, int l_max, const double* c1, const double* c2, int64_
       s2[x * nr + y] += f.b; s2[y * nr + x] += f.b;
       k2[x * nr + y] += f.b;
     }
+    // the columns of a tile in the order of their expected size, largest last (the kernel
+    // sums them plainly, and a partial sum rounds by its size): A_{n 0 0} counts the
+    // neighbours and is some five times any other A, and A of small n are the largest
+    auto size_n = [&](int c) {
+      auto of = [&](int l) { return l == 0 ? 5 : 1; };
+      if (c >= nc + na) return std::make_pair(50, 0);   // the constant 1
+      if (c >= nc) return std::make_pair(8 * of(L), -(c - nc + 1));
+      const int p = slots[c][0], q = slots[c][1];
+      return std::make_pair(of(lq(p)) * of(lq(q)), -(nq(p) + nq(q)));
+    };
+    auto before = [&](int x, int y) { return size_n(x) < size_n(y); };
     struct Tile { int row, rows; std::vector<int> cols[2]; };   // columns of S (both channels), of K2
     std::vector<Tile> tiles;
     for (int r0 = 0; r0 < nr; r0 += kQuadTile) {
@@ -441,6 +453,7 @@ bool build_quad(int n_max, int l_max, const double* c1, const double* c2, int64_
           }
           if (any) t.cols[pass].push_back(c);
         }
+        std::stable_sort(t.cols[pass].begin(), t.cols[pass].end(), before);
         const size_t unit = pass == 0 ? 2 : 4;   // columns per 64 bytes of values
         while (t.cols[pass].size() % unit) t.cols[pass].push_back(-1);
       }
