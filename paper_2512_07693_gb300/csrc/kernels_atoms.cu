@@ -1076,6 +1076,8 @@ __global__ void __launch_bounds__(kBlock, 3) k_pass2(Args<T> a) {
     T dv = T(0), dl = T(0), wb = T(1);
     if (PAPER) {
       wb = T(1) + u.wbar;   // the atom's own term, w(0) = 1
+      // (two atoms at one place, r = NaN in float32: the clamped taper lost it, zeta did not)
+      if (sizeof(T) == 4 && a.zeta[i] != a.zeta[i]) wb = a.zeta[i];
       dv = (a.g[i] + u.S) / wb - a.k.sw_d0;
       lam = ftrans_c(dv, a.k.sw_d_lo, a.k.sw_d_hi, a.k.sw_inv_d, &dl);
     } else {

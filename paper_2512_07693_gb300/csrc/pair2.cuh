@@ -39,15 +39,9 @@ __device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
 }
 // a - b, exactly rounded (the product b * -1 is exact)
 __device__ __forceinline__ F2 sub2(F2 a, F2 b) { return fma2(b, f2(-1.f), a); }
-// to [-1, 1]; a NaN (the distance of two atoms at one place) stays one, as in ftrans
-__device__ __forceinline__ float clamp_nan(float x) {
-  float r;
-  asm("{.reg .f32 t; max.NaN.f32 t, %1, 0fBF800000; min.NaN.f32 %0, t, 0f3F800000;}" : "=f"(r) : "f"(x));
-  return r;
-}
-__device__ __forceinline__ F2 clamp2(F2 a) {
+__device__ __forceinline__ F2 clamp2(F2 a) {   // to [-1, 1]
   const float2 v = f2_get(a);
-  return f2(clamp_nan(v.x), clamp_nan(v.y));
+  return f2(fminf(1.f, fmaxf(-1.f, v.x)), fminf(1.f, fmaxf(-1.f, v.y)));
 }
 // exp(x) as 2^(x log2 e) on the hardware's base-2 exponential
 __device__ __forceinline__ F2 exp2x(F2 x) {
@@ -67,7 +61,7 @@ __device__ __forceinline__ F2 rsqrt2(F2 x) {
 
 // The quintic taper f_trans at r (Eq. S1, in the factored form of ftrans), without
 // its two early returns: t clamped to [-1, 1] gives 1 and 0 exactly, and a zero
-// derivative, at the ends.  c = lo + hi, iw = 1 / (hi - lo).
+// derivative, at the ends (and 0 for a NaN).  c = lo + hi, iw = 1 / (hi - lo).
 __device__ __forceinline__ F2 taper_t(F2 r, F2 c, F2 iw) { return clamp2(mul2(fma2(f2(-2.f), r, c), iw)); }
 __device__ __forceinline__ F2 taper_f(F2 t) {
   const F2 p = add2(f2(1.f), t);
