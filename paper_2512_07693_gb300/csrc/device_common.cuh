@@ -18,9 +18,11 @@ template <typename T> struct V3 { T x, y, z; };
 // so that the next kernel in the stream may be scheduled while this one finishes
 // (launch_pdl).  Each calls pdl_begin() before its first memory access: it waits
 // until the previous kernel has completed and its writes are visible, then lets
-// its own dependent launch begin.  Waits end when the previous grid ends.
+// its own dependent launch begin.  Waits end when the previous grid ends.  (A kernel
+// that only calls pdl_wait() lets it begin when its own blocks have ended.)
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_begin() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_wait();
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
