@@ -115,11 +115,13 @@ typedef struct apip_params {
   int32_t ace_group;         /* compacted atoms per ACE thread block, or 0 = automatic.
                                 Body order <= 3 (streamed): 4, 8 or 32 (automatic: 2, 4, 8
                                 or 32 by the number of compacted atoms).  Body order 4
-                                (pool): 1, 2, 4 or 8 (automatic in float64: the largest
-                                whose two per-atom pools leave room for two resident blocks
-                                per SM; in float32 the quadratic evaluation, 8).  A group the evaluation does not provide, or whose
-                                shared memory does not fit, is rejected by apip_create
-                                (APIP_ERR_ARG). */
+                                (pool): 1, 2, 4 or 8 (automatic: the largest whose two
+                                per-atom pools leave room for two resident blocks per SM;
+                                in float32, where that is 1 or 2, the quadratic evaluation
+                                of 8, on a basis of up to 32 768 functions for more than
+                                some 100 or 200 compacted atoms).  A group the
+                                evaluation does not provide, or whose shared memory does
+                                not fit, is rejected by apip_create (APIP_ERR_ARG). */
   double ace_rc, ace_rc_width, ace_eps, ace_a_scale;
   const double* ace_c1;      /* host, ace_n_basis entries (copied) */
   const double* ace_c2;      /* host, ace_n_basis entries (copied) */

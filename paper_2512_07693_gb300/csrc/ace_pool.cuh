@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(kAceThreads) k_ace_pool(Args<T> a, AceDev<T> t
   T* A = X + KA;                           // A[c * KA + k] = X[(1 + c) * KA + k]
   T* W = G + KA;                           // omega, same layout as A
   const int count = a.counts[0];
-  const int ngroups = (count + KA - 1) / KA;
+  const int ngroups = count <= t.split ? (count + KA - 1) / KA : 0;   // (else the quadratic kernel's)
   double e_part = 0.0;
 
   for (int grp = blockIdx.x; grp < ngroups; grp += gridDim.x) {

@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(kQuadThreads, 1) k_ace_quad(Args<float> a, Ace
   float* X = red + 2 * (NT / 32) * NAT;                  // X_L, then dE/dX_L (step 1 stages R, Y there)
   float* Y = X + t.qrows * NAT;
   const int count = a.counts[0];
-  const int ngroups = (count + NAT - 1) / NAT;
+  const int ngroups = count > t.split ? (count + NAT - 1) / NAT : 0;   // (else the pool kernel's)
   double e_part = 0.0;
 
   for (int grp = blockIdx.x; grp < ngroups; grp += gridDim.x) {

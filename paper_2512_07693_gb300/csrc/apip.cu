@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -350,16 +351,13 @@ AceDev<T> ace_dev(apip_ctx* c) {
     t.group = c->ace_group;
     return t;
   }
-  if (t.kind == kAceQuad) {
-    t.qhdr = reinterpret_cast<const int4*>(b + c->ace_off[0]);
-    t.qmap = reinterpret_cast<const short*>(b + c->ace_off[1]);
-    t.qtile = reinterpret_cast<const int4*>(b + c->ace_off[2]);
-    t.qval = reinterpret_cast<const ulonglong2*>(b + c->ace_off[3]);
-    t.qcol = reinterpret_cast<const uint32_t*>(b + c->ace_off[4]);
-    t.qrows = c->ace_qrows;
-    t.group = c->ace_group;
-    return t;
-  }
+  t.qhdr = reinterpret_cast<const int4*>(b + c->ace_off[8]);
+  t.qmap = reinterpret_cast<const short*>(b + c->ace_off[9]);
+  t.qtile = reinterpret_cast<const int4*>(b + c->ace_off[10]);
+  t.qval = reinterpret_cast<const ulonglong2*>(b + c->ace_off[11]);
+  t.qcol = reinterpret_cast<const uint32_t*>(b + c->ace_off[12]);
+  t.qrows = c->ace_qrows;
+  t.split = t.kind == kAceQuad ? c->ace_split : INT_MAX;
   t.comp = reinterpret_cast<const uint2*>(b + c->ace_off[0]);
   t.gent = reinterpret_cast<const Ent<T>*>(b + c->ace_off[1]);
   t.frec = reinterpret_cast<const Rec<T>*>(b + c->ace_off[2]);
@@ -412,12 +410,19 @@ void force_pipeline(apip_ctx* c, Args<T>& a, cudaStream_t s) {
   { NvtxRange nv("apip.pass1"); Phase ph(c, APIP_PHASE_PASS1, 1, s); pass1<T>(a, s); }
   { NvtxRange nv("apip.pass2"); Phase ph(c, APIP_PHASE_PASS2, a.det ? 3 : 1, s); launch_pass2<T>(a, s);
     if (a.force_mix) launch_fm_buffer<T>(a, s); }
-  { NvtxRange nv("apip.ace"); Phase ph(c, APIP_PHASE_ACE, 1, s); const AceDev<T> t = ace_dev<T>(c);
-    if (t.kind == kAceStreamed) launch_ace_stream<T>(a, t, c->ace_blocks, s);
-    else if constexpr (sizeof(T) == 4) {
-      if (t.kind == kAceQuad) launch_ace_quad(a, t, c->ace_blocks, s);
-      else launch_ace_pool<T>(a, t, c->ace_blocks, s);
-    } else launch_ace_pool<T>(a, t, c->ace_blocks, s); }
+  { NvtxRange nv("apip.ace"); Phase ph(c, APIP_PHASE_ACE, (c->ace_blocks > 0) + (c->quad_blocks > 0), s); const AceDev<T> t = ace_dev<T>(c);
+    if (t.kind == kAceStreamed) {
+      launch_ace_stream<T>(a, t, c->ace_blocks, s);
+    } else {
+      if (c->ace_blocks > 0) launch_ace_pool<T>(a, t, c->ace_blocks, s);
+      if constexpr (sizeof(T) == 4) {
+        if (t.kind == kAceQuad) {
+          Args<float> q = a;   // its energy partials follow the pool kernel's
+          q.n_part_p1 += c->ace_blocks;
+          launch_ace_quad(q, t, c->quad_blocks, s);
+        }
+      }
+    } }
   if (a.lam_mode == APIP_LAM_PAPER && a.grad_lambda) {
     NvtxRange nv("apip.csp");
     Phase ph(c, APIP_PHASE_CSP, 1, s);
@@ -445,7 +450,7 @@ apip_status energy_forces_t(apip_ctx* c, const double* pos, const int32_t* id, i
   force_pipeline<T>(c, a, s);
   if (e_total) {
     Phase ph(c, APIP_PHASE_REDUCE, 1, s);
-    launch_final(c->partials, a.n_part_p1 + c->ace_blocks, e_total, nullptr, nullptr, 0, nullptr,
+    launch_final(c->partials, a.n_part_p1 + c->ace_blocks + c->quad_blocks, e_total, nullptr, nullptr, 0, nullptr,
                  c->flags, c->counts, nullptr, c->cell_count, c->ncell, c->e_scratch, c->counts + 2, s);
   }
   if (a.ind_on) launch_ind_work(c->ind_acc, 0.0, a.det, s);
@@ -493,7 +498,7 @@ apip_status verlet_t(apip_ctx* c, double* pos, double* vel, double* force, const
   set_view<T>(a, c);
   mark_atom_count(c, n, s);
   const int ntb = nblk(n);
-  const int n_part = a.n_part_p1 + c->ace_blocks;
+  const int n_part = a.n_part_p1 + c->ace_blocks + c->quad_blocks;
   // without thermo output the step needs no reduction at all: the energy partials
   // are left unread and the ACE kernel clears the rebuild flag
   double* tp = thermo ? c->thermo_part : nullptr;
@@ -547,11 +552,10 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
   ctx->p.ace_c2 = nullptr;
   ctx->nmax = n_atoms_max;
   ctx->r_list = std::max(std::max(p->eam_rc, p->ace_rc), p->sw_r_w) + p->skin;
-  // body order <= 3: streamed couplings; body order 4: in float32 the quadratic
-  // evaluation, which has its own atoms per block, in float64 or with a group size
-  // asked for the coupling pool
+  // body order <= 3: streamed couplings; body order 4: the coupling pool, in float32
+  // without a group size asked for also the quadratic evaluation
   const bool streamed = p->ace_nu_max <= 3;
-  const bool quad = !streamed && p->precision == APIP_FP32 && p->ace_group == 0;
+  bool quad = false;
   HostQuad hq;
   HostAce tab;
   HostStream st;
@@ -567,12 +571,7 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
     delete ctx;
     return APIP_ERR_ARG;
   }
-  if (quad && !(build_quad(p->ace_n_max, p->ace_l_max, ctx->ace_c1.data(), ctx->ace_c2.data(), nb, &hq, &why) &&
-                validate_quad(hq, &why))) {
-    delete ctx;
-    return APIP_ERR_ARG;
-  }
-  ctx->ace_kind = streamed ? kAceStreamed : (quad ? kAceQuad : kAcePool);
+  ctx->ace_kind = streamed ? kAceStreamed : kAcePool;
   const int nA = p->ace_n_max * (p->ace_l_max + 1) * (p->ace_l_max + 1);
   auto fail_create = [&](cudaError_t e) {
     free_all(ctx);
@@ -605,12 +604,7 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
       return streamed ? ace_stream_occupancy<double>(t) : ace_pool_occupancy<double>(t);
     };
     int group = p->ace_group, occ = 0;
-    if (quad) {
-      AceDev<float> t{};
-      t.l_max = p->ace_l_max; t.nA = nA; t.qrows = hq.rows;
-      group = kQuadAtoms;
-      occ = ace_quad_occupancy(t);
-    } else if (streamed) {
+    if (streamed) {
       if (group == 0 || group == 4 || group == 8 || group == 32) occ = occ_of(group);
       if (group == 0) {   // 32 atoms per block cost a large float64 basis its second resident block
         const bool adaptive = p->lam_mode == APIP_LAM_PAPER || p->lam_mode == APIP_LAM_LEARNED;
@@ -636,7 +630,33 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
       return APIP_ERR_ARG;
     }
     ctx->ace_group = group;
-    ctx->ace_blocks = std::max(1, sms) * occ;
+    ctx->ace_blocks = ctx->sms * occ;
+    // Body order 4 in float32: the quadratic kernel where the pools leave room for at
+    // most two atoms per block (2600 compacted atoms, whole call: basis 4/2 with pools of
+    // 8: pool kernel 77, quadratic 163 us; 4/4 with 4: 409 and 461; 6/3 with 4: 462 and
+    // 458; 7/3 with 2: 845 and 594; 8/4 with 1: 6400 and 1511).  On a basis of up to
+    // 32 k functions one of its blocks takes longer than a pool block (5/4: 222 and 178
+    // us, 7/3: 209 and 188, 6/4: 288 and 257; 8/3, 35 756: 255 and 264), so that there
+    // the pool kernel takes the calls whose groups have an SM each (up to two blocks for
+    // three SMs: beyond, some share one: 7/3, 250 atoms: 230 and 220).
+    if (!streamed && f32 && p->ace_group == 0 && group <= 2) {
+      if (!(build_quad(p->ace_n_max, p->ace_l_max, ctx->ace_c1.data(), ctx->ace_c2.data(), nb, &hq, &why) &&
+            validate_quad(hq, &why))) {
+        delete ctx;
+        return APIP_ERR_ARG;
+      }
+      AceDev<float> t{};
+      t.l_max = p->ace_l_max; t.nA = nA; t.qrows = hq.rows;
+      const int occ_q = ace_quad_occupancy(t);
+      cudaGetLastError();
+      quad = occ_q >= 1;
+      if (quad) {
+        ctx->ace_kind = kAceQuad;
+        ctx->ace_split = nb <= 32768 ? ctx->sms * group * 2 / 3 : 0;
+        if (ctx->ace_split == 0) ctx->ace_blocks = 0;
+        ctx->quad_blocks = ctx->sms * occ_q;
+      }
+    }
   }
   const size_t N = (size_t)n_atoms_max;
   const size_t es = esize(ctx);
@@ -681,7 +701,7 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
   // smaller blocks), or a small system's with several threads per atom (atom_lanes)
   const int p1 = (int)std::max<int64_t>(std::max(nblk(n_atoms_max), 4 * ctx->sms + 1),
                                         (n_atoms_max + kLearnedBlock - 1) / kLearnedBlock);
-  APIP_ALLOC(ctx->partials, sizeof(double) * (p1 + ctx->ace_blocks));
+  APIP_ALLOC(ctx->partials, sizeof(double) * (p1 + ctx->ace_blocks + ctx->quad_blocks));
   APIP_ALLOC(ctx->thermo_part, sizeof(double) * 4 * p1);
   APIP_ALLOC(ctx->e_scratch, sizeof(double) * kFinalScratch);
   APIP_ALLOC(ctx->ind_acc, sizeof(double) * 3);
@@ -767,21 +787,22 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
                6 * (int64_t)st.pkey.size();
   } else {
     if (quad) {
-      put(0, hq.hdr.data(), sizeof(int) * hq.hdr.size());
-      put(1, hq.map.data(), sizeof(short) * hq.map.size());
-      put(2, hq.tile.data(), sizeof(int) * hq.tile.size());
-      put(3, hq.val.data(), sizeof(float) * hq.val.size());
-      put(4, hq.col.data(), sizeof(uint32_t) * hq.col.size());
+      put(8, hq.hdr.data(), sizeof(int) * hq.hdr.size());
+      put(9, hq.map.data(), sizeof(short) * hq.map.size());
+      put(10, hq.tile.data(), sizeof(int) * hq.tile.size());
+      put(11, hq.val.data(), sizeof(float) * hq.val.size());
+      put(12, hq.col.data(), sizeof(uint32_t) * hq.col.size());
       ctx->ace_qrows = hq.rows;
-    } else {
-    put(0, tab.comp.data(), sizeof(uint32_t) * tab.comp.size());
-    put_ent(1, tab.gkey, tab.gval);
-    put_rec(2, tab.fkey, &tab.flen, tab.f1, tab.f2);
-    put(3, tab.qrow.data(), sizeof(int) * tab.qrow.size());
-    put_rec(4, tab.rkey, nullptr, tab.r1, tab.r2);
-    put_ent(5, tab.bkey, tab.bval);
-    put(6, tab.poff.data(), sizeof(int) * tab.poff.size());
-    put(7, tab.tpiece.data(), sizeof(int) * tab.tpiece.size());
+    }
+    if (ctx->ace_blocks > 0) {
+      put(0, tab.comp.data(), sizeof(uint32_t) * tab.comp.size());
+      put_ent(1, tab.gkey, tab.gval);
+      put_rec(2, tab.fkey, &tab.flen, tab.f1, tab.f2);
+      put(3, tab.qrow.data(), sizeof(int) * tab.qrow.size());
+      put_rec(4, tab.rkey, nullptr, tab.r1, tab.r2);
+      put_ent(5, tab.bkey, tab.bval);
+      put(6, tab.poff.data(), sizeof(int) * tab.poff.size());
+      put(7, tab.tpiece.data(), sizeof(int) * tab.tpiece.size());
     }
     ctx->ace_nC = tab.nC;
     ctx->ace_npool = tab.npool;
@@ -800,9 +821,9 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
     info[10] = 3 * info[2] + 2 * info[4] + 4 * info[3] + 4 * info[5] + 3 * info[6];
   }
   // (streamed without a group asked for: the group of a large system)
-  ctx->ace_info[7] = ctx->ace_group != 0 ? ctx->ace_group
+  ctx->ace_info[7] = quad ? kQuadAtoms : ctx->ace_group != 0 ? ctx->ace_group
                      : p->lam_mode == APIP_LAM_PAPER || p->lam_mode == APIP_LAM_LEARNED ? 8 : 32;
-  ctx->ace_info[8] = ctx->ace_blocks;
+  ctx->ace_info[8] = quad ? ctx->quad_blocks : ctx->ace_blocks;
   ctx->ace_info[9] = streamed ? 1 : 0;
   APIP_ALLOC(ctx->ace_tab, host.size());
 #undef APIP_ALLOC
@@ -831,10 +852,9 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
     gaunt_fill(gv.data());
     e = p->precision == APIP_FP64 ? ace_stream_set_consts<double>(norms, nn, gv.data())
                                   : ace_stream_set_consts<float>(norms, nn, gv.data());
-  } else if (quad) {
-    e = ace_quad_set_consts(norms, nn);
   } else {
     e = p->precision == APIP_FP64 ? ace_pool_set_norms<double>(norms, nn) : ace_pool_set_norms<float>(norms, nn);
+    if (e == cudaSuccess && quad) e = ace_quad_set_consts(norms, nn);
   }
   if (e != cudaSuccess) return fail_create(e);
   if (p->precision == APIP_FP64 && (e = exp_table_set()) != cudaSuccess) return fail_create(e);

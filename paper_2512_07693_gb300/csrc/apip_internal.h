@@ -117,6 +117,7 @@ struct AceDev {
   const ulonglong2* qval;       // values
   const uint32_t* qcol;         // columns as offsets of their rows in X_L
   int qrows;                    // most values of X_L per atom
+  int split;                    // the pool kernel takes the calls with up to this many atoms, the quadratic kernel the others
   int group;                    // compacted atoms per thread block (streamed: 0 = by their number, on the device)
   int top;                      // ... the largest of these, 8 or 32
   int sms;                      // SMs of the device
@@ -227,7 +228,7 @@ struct apip_ctx {
   double* thermo_part = nullptr;  // [blocks][4] KE, px, py, pz
   double* e_scratch = nullptr;    // [kFinalScratch] per-warp sums of k_final
   int n_part = 0;
-  int ace_blocks = 0;
+  int ace_blocks = 0, quad_blocks = 0;   // of the streamed or pool kernel, of the quadratic kernel
 
   // phase timing (apip_profile)
   bool prof = false;
@@ -240,8 +241,9 @@ struct apip_ctx {
   // ACE tables (element size = precision): one device buffer, sub-arrays at
   // the byte offsets ace_off (order of AceDev's pointers)
   void* ace_tab = nullptr;
-  size_t ace_off[8] = {};
+  size_t ace_off[13] = {};
   int ace_qrows = 0;
+  int ace_split = 0;           // (quadratic evaluation) see AceDev::split
   int ace_nf = 0, ace_npc = 0, ace_nC = 0, ace_npool = 0;
   int ace_group = 1;           // (streamed: 0 = chosen on the device)
   int ace_top = 32;            // ... up to this many
