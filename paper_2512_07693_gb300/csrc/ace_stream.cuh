@@ -369,83 +369,127 @@ __device__ __forceinline__ void stream_body(const Args<T>& a, const AceDev<T>& t
   block_energy<T, NAT>(a, g, e_part);
 }
 
-// Atoms per block (t.group, or by the number of compacted atoms where it is 0).  A
-// block's time is a serial chain over its slices' couplings, shorter with fewer atoms
-// (hence more slices): float32 about 30, 38, 47 and 105 us for 2, 4, 8 and 32, but the
-// table reads and the sums over the slices are per block, so that large counts want
-// large groups.  So: 2 while each SM has at most one block, 4 for one round of the
-// resident blocks, 8 for two rounds, 32 beyond (with an adaptive switch only where
-// that leaves as many blocks resident: t.top) (measured for every group at 100 to
-// 79 k compacted atoms in both precisions; whole call at 2000, 1 % of them
-// compacted: 65 -> 48 us, in float64 481 -> 295 us; all of them, 8 instead of 32:
-// 125 -> 65 us and 1069 -> 787 us).
-template <typename T, typename K, int LMAX>
+// Atoms per block where no group is asked for, by the number of compacted atoms (r: the
+// blocks that are resident).  A block's time is a serial chain over its slices'
+// couplings, shorter with fewer atoms (hence more slices), but the table reads and the
+// sums over the slices are per block, so that large counts want large groups: 2 and 4
+// for one round of the resident blocks, 8 for two rounds, 32 beyond (whole float32 call
+// on 8192 atoms, basis 6/3, groups of 2, 4, 8, 32: 608 compacted 51, 59, 68, 140 us;
+// 1216: 71, 62, 73, 141; 2432: 112, 92, 77, 140; 4864: 192, 152, 122, 159; 8000: 308,
+// 239, 201, 163).
+// In float64 blocks that share an SM take half as long again, which tells on bases of
+// some hundred couplings and more: there first the smallest group whose blocks have an
+// SM each (two blocks for three SMs: beyond, some share one; 6/3: 152 compacted 387, 431,
+// 551, 1172 us; 400: 500, 445, 561, 1176; 700: 699, 633, 565, 1174; 1216: 819, 641, 862,
+// 1177; 2432: 1450, 1107, 888, 1176; 4864: 2681, 2045, 1611, 2112).
+// many: above 600 couplings with l_max = 4 a second round of 8 is no better than 32 (8/4:
+// 2600 compacted: 588 and 548 us, float64 4849 and 4099; 6/4: 313 and 300).
+template <typename T>
+__device__ __forceinline__ int stream_group(const AceDev<T>& t, int count, int r, bool many) {
+  if (sizeof(T) == 8 && t.ncpl >= 300) {
+    const int alone = t.sms * 2 / 3;
+    if (count <= 8 * alone) return count <= 2 * alone ? 2 : count <= 4 * alone ? 4 : 8;
+  } else if (count <= 2 * r) {
+    return 2;
+  }
+  return count <= 4 * r ? 4 : count <= (many ? 8 : 16) * r || t.top == 8 ? 8 : 32;
+}
+
+// GROUP atoms per block, or (0) as many as stream_group says, all in one kernel.  With
+// l_max = 4 that kernel's code came out slower than the kernels of one group (8/4,
+// float32, 4 atoms per block: 424 and 262 us; 4/4: 90 and 85), so for more than 600
+// couplings there each group's kernel is launched in turn and all but one find that
+// the count is not theirs (3 us each: 1/4, 152 atoms: 70 -> 74 us).
+template <typename T, typename K, int LMAX, int GROUP>
 __global__ void __launch_bounds__(kAceThreads, 2) k_ace_stream(Args<T> a, AceDev<T> t) {
-  pdl_begin();
+  if (GROUP != 0 && t.group == 0) pdl_wait();   // (one of several: the next one's blocks are not to be let in beside these)
+  else pdl_begin();
   // every list-build kernel of this call has completed: block 0 clears the
   // trigger (and, after a build, the binning counts) for the next step
   if (blockIdx.x == 0) end_list_build(a.flags, a.cell_count, a.ncell);
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ __align__(16) unsigned char group[sizeof(AceGroup<T, 32>)];
-  int nat = t.group;
-  if (nat == 0) {
-    const int count = a.counts[0], r = (int)gridDim.x;
-    nat = count <= 2 * t.sms ? 2 : count <= 4 * r ? 4 : count <= 16 * r || t.top == 8 ? 8 : 32;
+  __shared__ __align__(16) unsigned char group[sizeof(AceGroup<T, GROUP == 0 ? 32 : GROUP>)];
+  if constexpr (GROUP != 0) {
+    if (t.group != 0 || stream_group(t, a.counts[0], t.slots, true) == GROUP)
+      stream_body<T, K, LMAX, GROUP>(a, t, smem_raw, group);
+    else if (threadIdx.x == 0) a.partials[a.n_part_p1 + blockIdx.x] = 0.0;
+  } else {
+    switch (stream_group(t, a.counts[0], (int)gridDim.x, false)) {
+      case 2: stream_body<T, K, LMAX, 2>(a, t, smem_raw, group); break;
+      case 4: stream_body<T, K, LMAX, 4>(a, t, smem_raw, group); break;
+      case 8: stream_body<T, K, LMAX, 8>(a, t, smem_raw, group); break;
+      default: stream_body<T, K, LMAX, 32>(a, t, smem_raw, group); break;
+    }
   }
-  switch (nat) {
-    case 2: stream_body<T, K, LMAX, 2>(a, t, smem_raw, group); break;
-    case 4: stream_body<T, K, LMAX, 4>(a, t, smem_raw, group); break;
-    case 8: stream_body<T, K, LMAX, 8>(a, t, smem_raw, group); break;
-    default: stream_body<T, K, LMAX, 32>(a, t, smem_raw, group); break;
+}
+
+// Shared memory of a launch: of GROUP, or of the largest group the kernel may choose
+// (t.top).
+template <typename T, int LMAX, int GROUP>
+size_t stream_smem(const AceDev<T>& t) {
+  if constexpr (GROUP != 0) {
+    return ace_stream_smem<T, LMAX, GROUP>(t.nA);
+  } else {
+    const size_t few = std::max({ace_stream_smem<T, LMAX, 2>(t.nA), ace_stream_smem<T, LMAX, 4>(t.nA),
+                                 ace_stream_smem<T, LMAX, 8>(t.nA)});
+    return t.top == 8 ? few : std::max(few, ace_stream_smem<T, LMAX, 32>(t.nA));
   }
 }
 
-// Shared memory of a launch: of the group asked for, else of the largest one the kernel
-// may choose (t.top).
-template <typename T, int LMAX>
-size_t stream_smem_of(const AceDev<T>& t) {
-  const size_t m4 = ace_stream_smem<T, LMAX, 4>(t.nA), m8 = ace_stream_smem<T, LMAX, 8>(t.nA);
-  const size_t m32 = ace_stream_smem<T, LMAX, 32>(t.nA);
-  if (t.group != 0) return t.group == 4 ? m4 : t.group == 8 ? m8 : m32;
-  const size_t few = std::max(ace_stream_smem<T, LMAX, 2>(t.nA), std::max(m4, m8));
-  return t.top == 8 ? few : std::max(few, m32);
-}
-
-template <typename T, typename K, int LMAX>
-void launch_stream_lk(const Args<T>& a, const AceDev<T>& t, int blocks, cudaStream_t s) {
-  const size_t bytes = stream_smem_of<T, LMAX>(t);
-  cudaFuncSetAttribute(k_ace_stream<T, K, LMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  launch_pdl(k_ace_stream<T, K, LMAX>, blocks, kAceThreads, bytes, s, a, t);
-}
-
-template <typename T, typename K, int LMAX>
-int occupancy_stream_lk(const AceDev<T>& t) {
-  const size_t bytes = stream_smem_of<T, LMAX>(t);
+template <typename T, typename K, int LMAX, int GROUP>
+int stream_l(const Args<T>* a, const AceDev<T>& t, int blocks, cudaStream_t s, bool query) {
+  const size_t bytes = stream_smem<T, LMAX, GROUP>(t);
+  auto kernel = k_ace_stream<T, K, LMAX, GROUP>;
+  if (!query) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    launch_pdl(kernel, blocks, kAceThreads, bytes, s, *a, t);
+    return 0;
+  }
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (bytes + (size_t)1024 > (size_t)optin) return 0;
-  if (cudaFuncSetAttribute(k_ace_stream<T, K, LMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)bytes) != cudaSuccess)
-    return 0;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return 0;
   int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_ace_stream<T, K, LMAX>, kAceThreads, bytes) !=
-      cudaSuccess)
-    return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, kAceThreads, bytes) != cudaSuccess) return 0;
   return occ;
 }
 
+// launch, or occupancy query (resident blocks per SM, 0 if it does not fit), of the kernel
+// of `group` atoms per block (0: the one that chooses)
+template <typename T, typename K, int LMAX>
+int stream_g(const Args<T>* a, const AceDev<T>& t, int group, int blocks, cudaStream_t s, bool query) {
+  switch (group) {
+    case 0: return stream_l<T, K, LMAX, 0>(a, t, blocks, s, query);
+    case 2: if constexpr (LMAX == 4) return stream_l<T, K, LMAX, 2>(a, t, blocks, s, query); else return 0;
+    case 4: return stream_l<T, K, LMAX, 4>(a, t, blocks, s, query);
+    case 8: return stream_l<T, K, LMAX, 8>(a, t, blocks, s, query);
+    case 32: return stream_l<T, K, LMAX, 32>(a, t, blocks, s, query);
+    default: return 0;
+  }
+}
+
 template <typename T, typename K>
-int stream_dispatch(const Args<T>* a, const AceDev<T>& t, int blocks, cudaStream_t s, bool query) {
+int stream_dispatch(const Args<T>* a, const AceDev<T>& t, int group, int blocks, cudaStream_t s, bool query) {
   switch (t.l_max) {
-#define APIP_CASE(L)                                           \
-  case L:                                                      \
-    if (query) return occupancy_stream_lk<T, K, L>(t);         \
-    launch_stream_lk<T, K, L>(*a, t, blocks, s);               \
-    return 0;
-    APIP_CASE(0) APIP_CASE(1) APIP_CASE(2) APIP_CASE(3)
-    default: APIP_CASE(4)
-#undef APIP_CASE
+    case 0: return stream_g<T, K, 0>(a, t, group, blocks, s, query);
+    case 1: return stream_g<T, K, 1>(a, t, group, blocks, s, query);
+    case 2: return stream_g<T, K, 2>(a, t, group, blocks, s, query);
+    case 3: return stream_g<T, K, 3>(a, t, group, blocks, s, query);
+    default: return stream_g<T, K, 4>(a, t, group, blocks, s, query);
+  }
+}
+
+template <typename T, typename K>
+void stream_launch(const Args<T>& a, const AceDev<T>& t, cudaStream_t s) {
+  if (t.grid[1] == 0) {
+    stream_dispatch<T, K>(&a, t, t.group, t.grid[0], s, false);
+    return;
+  }
+  Args<T> b = a;   // each kernel's energy partials behind those of the one before
+  for (int q = 0; q < 4; ++q) {
+    stream_dispatch<T, K>(&b, t, kStreamGroups[q], t.grid[q], s, false);
+    b.n_part_p1 += t.grid[q];
   }
 }
 

@@ -349,6 +349,8 @@ AceDev<T> ace_dev(apip_ctx* c) {
     t.npart = c->ace_npart;
     t.cfirst = reinterpret_cast<const Rec<T>*>(b + c->ace_off[3]);
     t.group = c->ace_group;
+    for (int q = 0; q < 4; ++q) t.grid[q] = c->ace_grid[q];
+    t.slots = c->ace_grid[2];
     return t;
   }
   t.qhdr = reinterpret_cast<const int4*>(b + c->ace_off[8]);
@@ -410,9 +412,9 @@ void force_pipeline(apip_ctx* c, Args<T>& a, cudaStream_t s) {
   { NvtxRange nv("apip.pass1"); Phase ph(c, APIP_PHASE_PASS1, 1, s); pass1<T>(a, s); }
   { NvtxRange nv("apip.pass2"); Phase ph(c, APIP_PHASE_PASS2, a.det ? 3 : 1, s); launch_pass2<T>(a, s);
     if (a.force_mix) launch_fm_buffer<T>(a, s); }
-  { NvtxRange nv("apip.ace"); Phase ph(c, APIP_PHASE_ACE, (c->ace_blocks > 0) + (c->quad_blocks > 0), s); const AceDev<T> t = ace_dev<T>(c);
+  { NvtxRange nv("apip.ace"); Phase ph(c, APIP_PHASE_ACE, c->ace_launches, s); const AceDev<T> t = ace_dev<T>(c);
     if (t.kind == kAceStreamed) {
-      launch_ace_stream<T>(a, t, c->ace_blocks, s);
+      launch_ace_stream<T>(a, t, s);
     } else {
       if (c->ace_blocks > 0) launch_ace_pool<T>(a, t, c->ace_blocks, s);
       if constexpr (sizeof(T) == 4) {
@@ -604,8 +606,15 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
       return streamed ? ace_stream_occupancy<double>(t) : ace_pool_occupancy<double>(t);
     };
     int group = p->ace_group, occ = 0;
-    if (streamed) {
-      if (group == 0 || group == 4 || group == 8 || group == 32) occ = occ_of(group);
+    if (streamed && group == 0 && p->ace_l_max == 4 && st.cpl.size() / 4 > 600) {
+      occ = 1;
+      for (int q = 0; q < 4; ++q) {
+        const int o = occ_of(kStreamGroups[q]);
+        occ = std::min(occ, o);
+        ctx->ace_grid[q] = ctx->sms * o;
+      }
+    } else if (streamed) {
+      occ = group == 2 ? 0 : occ_of(group);   // 0 for a group the kernel does not provide
       if (group == 0) {   // 32 atoms per block cost a large float64 basis its second resident block
         const bool adaptive = p->lam_mode == APIP_LAM_PAPER || p->lam_mode == APIP_LAM_LEARNED;
         ctx->ace_top = 8;
@@ -613,6 +622,7 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
         if (occ >= occ8 || (!adaptive && occ >= 1)) ctx->ace_top = 32;
         else occ = occ8;
       }
+      ctx->ace_grid[0] = ctx->sms * occ;
     } else if (group != 0) {
       occ = occ_of(group);   // 0 for a group the kernel does not provide
     } else {
@@ -631,6 +641,10 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
     }
     ctx->ace_group = group;
     ctx->ace_blocks = ctx->sms * occ;
+    if (streamed) {
+      ctx->ace_blocks = 0;
+      for (int b : ctx->ace_grid) ctx->ace_blocks += b;
+    }
     // Body order 4 in float32: the quadratic kernel where the pools leave room for at
     // most two atoms per block (2600 compacted atoms, whole call: basis 4/2 with pools of
     // 8: pool kernel 77, quadratic 163 us; 4/4 with 4: 409 and 461; 6/3 with 4: 462 and
@@ -658,6 +672,7 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
       }
     }
   }
+  ctx->ace_launches = streamed ? (ctx->ace_grid[1] > 0 ? 4 : 1) : (ctx->ace_blocks > 0) + (ctx->quad_blocks > 0);
   const size_t N = (size_t)n_atoms_max;
   const size_t es = esize(ctx);
   APIP_ALLOC(ctx->nnb, sizeof(int) * N);

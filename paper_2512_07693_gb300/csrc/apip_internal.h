@@ -84,6 +84,7 @@ template <typename T> struct alignas(sizeof(T) == 4 ? 8 : 16) Ent { T v; uint32_
 //    every function of that degree is an entry of a symmetric matrix S_L shared by
 //    all atoms: phi_c = sum_L 1/2 X_L . (S_L^c X_L).
 constexpr int kAcePool = 0, kAceStreamed = 1, kAceQuad = 2;
+constexpr int kStreamGroups[4] = {2, 4, 8, 32};   // atoms per block that the streamed evaluation chooses from
 constexpr int kQuadAtoms = 8;       // atoms per block of the quadratic evaluation
 constexpr int kQuadThreads = 384;   // its threads per block
 constexpr int kQuadTile = 4;        // rows of S_L per tile
@@ -120,6 +121,8 @@ struct AceDev {
   int split;                    // the pool kernel takes the calls with up to this many atoms, the quadratic kernel the others
   int group;                    // compacted atoms per thread block (streamed: 0 = by their number, on the device)
   int top;                      // ... the largest of these, 8 or 32
+  int grid[4];                  // streamed: blocks of the launch ([0]), or of the kernel of each of kStreamGroups
+  int slots;                    // ... resident blocks (of 8 atoms)
   int sms;                      // SMs of the device
 };
 
@@ -228,7 +231,8 @@ struct apip_ctx {
   double* thermo_part = nullptr;  // [blocks][4] KE, px, py, pz
   double* e_scratch = nullptr;    // [kFinalScratch] per-warp sums of k_final
   int n_part = 0;
-  int ace_blocks = 0, quad_blocks = 0;   // of the streamed or pool kernel, of the quadratic kernel
+  int ace_blocks = 0, quad_blocks = 0;   // of the streamed or pool kernel(s), of the quadratic kernel
+  int ace_launches = 1;        // ACE kernels per call
 
   // phase timing (apip_profile)
   bool prof = false;
@@ -247,6 +251,7 @@ struct apip_ctx {
   int ace_nf = 0, ace_npc = 0, ace_nC = 0, ace_npool = 0;
   int ace_group = 1;           // (streamed: 0 = chosen on the device)
   int ace_top = 32;            // ... up to this many
+  int ace_grid[4] = {};        // see AceDev::grid
   int ace_kind = 0, ace_npr = 0, ace_ncpl = 0, ace_npart = 0;
   int64_t ace_info[APIP_ACE_INFO_COUNT] = {};
 

@@ -313,7 +313,7 @@ cudaError_t ace_quad_set_consts(const double* norms, int count);
 void launch_ace_quad(const Args<float>& a, const AceDev<float>& ace, int blocks, cudaStream_t s);
 int ace_quad_occupancy(const AceDev<float>& ace);
 template <typename T> cudaError_t ace_stream_set_consts(const double* norms, int count, const double* gaunt);
-template <typename T> void launch_ace_stream(const Args<T>& a, const AceDev<T>& ace, int blocks, cudaStream_t s);
+template <typename T> void launch_ace_stream(const Args<T>& a, const AceDev<T>& ace, cudaStream_t s);
 template <typename T> int ace_stream_occupancy(const AceDev<T>& ace);
 
 }  // namespace apip

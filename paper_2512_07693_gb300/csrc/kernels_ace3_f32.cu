@@ -26,12 +26,12 @@ template <> cudaError_t ace_stream_set_consts<float>(const double* norms, int co
   return cudaMemcpyToSymbol(c_gaunt, gv.data(), sizeof(float) * kGauntTotal);
 }
 
-template <> void launch_ace_stream<float>(const Args<float>& a, const AceDev<float>& t, int blocks, cudaStream_t s) {
-  stream_dispatch<float, Consts>(&a, t, blocks, s, false);
+template <> void launch_ace_stream<float>(const Args<float>& a, const AceDev<float>& t, cudaStream_t s) {
+  stream_launch<float, Consts>(a, t, s);
 }
 
 template <> int ace_stream_occupancy<float>(const AceDev<float>& t) {
-  return stream_dispatch<float, Consts>(nullptr, t, 0, nullptr, true);
+  return stream_dispatch<float, Consts>(nullptr, t, t.group, 0, nullptr, true);
 }
 
 }  // namespace apip

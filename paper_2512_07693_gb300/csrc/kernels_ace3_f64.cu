@@ -26,12 +26,12 @@ template <> cudaError_t ace_stream_set_consts<double>(const double* norms, int c
   return cudaMemcpyToSymbol(c_gaunt, gv.data(), sizeof(double) * kGauntTotal);
 }
 
-template <> void launch_ace_stream<double>(const Args<double>& a, const AceDev<double>& t, int blocks, cudaStream_t s) {
-  stream_dispatch<double, Consts>(&a, t, blocks, s, false);
+template <> void launch_ace_stream<double>(const Args<double>& a, const AceDev<double>& t, cudaStream_t s) {
+  stream_launch<double, Consts>(a, t, s);
 }
 
 template <> int ace_stream_occupancy<double>(const AceDev<double>& t) {
-  return stream_dispatch<double, Consts>(nullptr, t, 0, nullptr, true);
+  return stream_dispatch<double, Consts>(nullptr, t, t.group, 0, nullptr, true);
 }
 
 }  // namespace apip

@@ -1063,16 +1063,14 @@ __device__ __forceinline__ Pass2Sums<double> pass2_sums(const Args<double>& a, i
 
 //
 // With several threads per atom the ACE kernel's blocks are let onto the SMs only when
-// those of this pass have ended (unless no atom can have lam > 0).  Let in before, they
-// go in twos and threes to the SMs that are free first while others stay empty, and an
-// ACE block beside another takes up to 1.5 times as long: 40 compacted atoms of 8192,
-// body order 4 on basis 7/3: 244 to 300 -> 190 us; float64: 472 -> 358 us; 27 k-atom
-// step 85.9 -> 83.5 us.  Without compacted atoms the later start costs 2 of 25 us; in a
-// large system it gains nothing (249 k atoms: 177 us either way) and costs 1.5 % with
-// the learned switch at 900 k atoms.
+// those of this pass have ended.  Let in before, they go in twos and threes to the SMs
+// that are free first while others stay empty, and an ACE block beside another takes up
+// to 1.5 times as long: 40 compacted atoms of 8192, body order 4 on basis 7/3: 244 to 300
+// -> 190 us; float64: 472 -> 358 us; 27 k-atom step 85.9 -> 83.5 us.  In a large system
+// it gains nothing (249 k atoms: 177 us either way).
 template <typename T, bool PAPER, int LANES>
 __global__ void __launch_bounds__(kBlock, 3) k_pass2(Args<T> a) {
-  if (LANES == 1 || (a.lam_mode == APIP_LAM_CONST0 && !a.lam_fixed)) pdl_begin();
+  if (LANES == 1) pdl_begin();
   else pdl_wait();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int g = LANES == 1 ? 0 : (int)(threadIdx.x % LANES);
