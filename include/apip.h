@@ -168,7 +168,13 @@ typedef struct apip_params {
 int64_t apip_ace_basis_size(int32_t n_max, int32_t l_max, int32_t nu_max);
 
 /* Create a context for up to n_atoms_max atoms.  Allocates all scratch (cells,
- * neighbour list, per-atom switch arrays, ACE tables) on the current device.
+ * neighbour list, per-atom switch arrays, ACE tables) on the current device: some
+ * 8 max_nb + 210 bytes per atom (192 in float64; the learned switch 128 more in
+ * float32), and 16 cell_cap + 4 per cell of the first box (later of the largest).  A
+ * float64 context without the learned switch takes 8 max_nb more per atom to keep
+ * the EAM pair terms of a call's first pass for its second, where that is no more than
+ * an eighth of the memory still free; it gives them back when the cells of a box do not
+ * fit, and then computes them twice.
  * Errors: APIP_ERR_ARG (bad parameters, or an ACE group that does not fit in
  * shared memory), APIP_ERR_CUDA (allocation). */
 apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** out);

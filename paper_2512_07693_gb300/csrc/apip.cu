@@ -135,6 +135,21 @@ apip_status check_params(const apip_params* p, std::string* why) {
   return APIP_OK;
 }
 
+// The cell arrays; where memory is short, the kept pair terms (optional) make room.
+// (cudaFree waits for the calls in flight.  A graph captured with them holds the old cell
+// arrays too, which set_geometry frees before it comes here.)
+cudaError_t alloc_cells(apip_ctx* c, void** ptr, size_t bytes) {
+  cudaError_t e = cudaMalloc(ptr, bytes);
+  if (e == cudaErrorMemoryAllocation && c->pair_keep) {
+    cudaGetLastError();
+    cudaFree(c->pair_keep);
+    c->pair_keep = nullptr;
+    c->pair_rows = 0;
+    e = cudaMalloc(ptr, bytes);
+  }
+  return e;
+}
+
 // Cell grid for a new box; marks the neighbour list for rebuild.
 apip_status set_geometry(apip_ctx* ctx, const double* box, cudaStream_t s) {
   if (!box) return fail(ctx, APIP_ERR_ARG, "box must not be NULL");
@@ -164,9 +179,10 @@ apip_status set_geometry(apip_ctx* ctx, const double* box, cudaStream_t s) {
     if (ctx->cell_q) cudaFree(ctx->cell_q);
     ctx->cell_count = nullptr;
     ctx->cell_q = nullptr;
-    APIP_CK(cudaMalloc(&ctx->cell_count, sizeof(int) * ncell));
+    ctx->ncell_alloc = 0;
+    APIP_CK(alloc_cells(ctx, (void**)&ctx->cell_count, sizeof(int) * ncell));
     APIP_CK(cudaMemsetAsync(ctx->cell_count, 0, sizeof(int) * ncell, s));
-    APIP_CK(cudaMalloc(&ctx->cell_q, sizeof(uint4) * (size_t)ncell * ctx->p.cell_cap));
+    APIP_CK(alloc_cells(ctx, (void**)&ctx->cell_q, sizeof(uint4) * (size_t)ncell * ctx->p.cell_cap));
     ctx->ncell_alloc = ncell;
   }
   ctx->ncell = ncell;
@@ -264,7 +280,7 @@ Args<T> make_args(apip_ctx* c, const double* pos, const int* id, int n, double* 
   a.r_scan2f = std::nextafter((float)(a.r_list2 * (1.0 + 4e-5)), INFINITY);
   a.lanes = atom_lanes(n, c->sms);
   a.pair_keep = static_cast<double2*>(c->pair_keep);
-  a.pair_rows = p.lam_mode == APIP_LAM_LEARNED ? 0 : c->pair_rows;   // (the learned pass 1 keeps none)
+  a.pair_rows = c->pair_rows;
   a.csp_rcut2 = p.csp_rcut * p.csp_rcut;
   a.pos = pos;
   a.id = id;
@@ -693,17 +709,6 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
   APIP_ALLOC(ctx->csp_owner, sizeof(int) * N);
   void** per_atom[] = {&ctx->zeta, &ctx->xi_p, &ctx->e_eam, &ctx->g, &ctx->wbar, &ctx->dd, &ctx->lam, &ctx->dlam, &ctx->e_ace};
   for (void** q : per_atom) APIP_ALLOC(*q, es * N);
-  if (p->precision == APIP_FP64) {
-    // pass 1's pair terms for pass 2: class 0 of the list (within the EAM cutoff) is
-    // less than half of it.  An entry beyond these rows is computed again, so is
-    // every entry where there is no room for them
-    ctx->pair_rows = (p->max_nb + 1) / 2;
-    if (cudaMalloc(&ctx->pair_keep, sizeof(double2) * N * ctx->pair_rows) != cudaSuccess) {
-      cudaGetLastError();
-      ctx->pair_keep = nullptr;
-      ctx->pair_rows = 0;
-    }
-  }
   APIP_ALLOC(ctx->cvec, sizeof(double) * N);
   APIP_ALLOC(ctx->ace_list, sizeof(int) * N);
   if (p->lam_mode == APIP_LAM_LEARNED) APIP_ALLOC(ctx->clist, sizeof(int) * N);
@@ -842,6 +847,21 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
   ctx->ace_info[9] = streamed ? 1 : 0;
   APIP_ALLOC(ctx->ace_tab, host.size());
 #undef APIP_ALLOC
+  if (p->precision == APIP_FP64 && p->lam_mode != APIP_LAM_LEARNED) {   // (the learned pass 1 keeps none)
+    // pass 1's pair terms for pass 2: class 0 of the list (within the EAM cutoff) is
+    // less than half of it.  An entry beyond these rows is computed again, so is
+    // every entry where there is no room for them: they come after everything that a
+    // context cannot do without, take no more than an eighth of what is then free, and
+    // make room for the cells of a box (alloc_cells)
+    const size_t rows = (size_t)(p->max_nb + 1) / 2;
+    size_t avail = 0, total = 0;
+    if (cudaMemGetInfo(&avail, &total) == cudaSuccess && sizeof(double2) * N * rows <= avail / 8 &&
+        cudaMalloc(&ctx->pair_keep, sizeof(double2) * N * rows) == cudaSuccess)
+      ctx->pair_rows = (int)rows;
+    else
+      ctx->pair_keep = nullptr;
+    cudaGetLastError();
+  }
   cudaError_t e = cudaMemcpy(ctx->ace_tab, host.data(), host.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(ctx->id2idx, 0xff, sizeof(int) * N);
   if (e == cudaSuccess) e = cudaMemset(ctx->csp, 0xff, sizeof(int) * N * kCspCap);
