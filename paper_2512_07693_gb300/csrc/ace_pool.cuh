@@ -173,42 +173,22 @@ __global__ void __launch_bounds__(kAceThreads) k_ace_pool(Args<T> a, AceDev<T> t
 }
 
 template <typename T, typename K, int LMAX, int KA>
-void launch_pool_lk(const Args<T>& a, const AceDev<T>& t, int blocks, cudaStream_t s) {
+int pool_l(const Args<T>* a, const AceDev<T>& t, int blocks, cudaStream_t s, bool query) {
   const size_t bytes = ace_pool_smem<T, LMAX, KA>(t.npool);
-  cudaFuncSetAttribute(k_ace_pool<T, K, LMAX, KA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  launch_pdl(k_ace_pool<T, K, LMAX, KA>, blocks, kAceThreads, bytes, s, a, t);
+  if (query) return resident_blocks(k_ace_pool<T, K, LMAX, KA>, kAceThreads, bytes);
+  launch_pdl(k_ace_pool<T, K, LMAX, KA>, blocks, kAceThreads, bytes, s, *a, t);
+  return 0;
 }
 
-// Resident blocks per SM for this pool size (0 if it does not fit).
-template <typename T, typename K, int LMAX, int KA>
-int occupancy_pool_lk(int npool) {
-  const size_t bytes = ace_pool_smem<T, LMAX, KA>(npool);
-  int dev = 0, optin = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (bytes + (size_t)1024 > (size_t)optin) return 0;
-  if (cudaFuncSetAttribute(k_ace_pool<T, K, LMAX, KA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) !=
-      cudaSuccess)
-    return 0;
-  int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_ace_pool<T, K, LMAX, KA>, kAceThreads, bytes) !=
-      cudaSuccess)
-    return 0;
-  return occ;
-}
-
-// launch (occ == nullptr) or occupancy query for (l_max, group)
+// launch, or occupancy query, for (l_max, group)
 template <typename T, typename K, int KA>
 int pool_k(const Args<T>* a, const AceDev<T>& t, int blocks, cudaStream_t s, bool query) {
   switch (t.l_max) {
-#define APIP_CASE(L)                                          \
-  case L:                                                     \
-    if (query) return occupancy_pool_lk<T, K, L, KA>(t.npool); \
-    launch_pool_lk<T, K, L, KA>(*a, t, blocks, s);            \
-    return 0;
-    APIP_CASE(0) APIP_CASE(1) APIP_CASE(2) APIP_CASE(3)
-    default: APIP_CASE(4)
-#undef APIP_CASE
+    case 0: return pool_l<T, K, 0, KA>(a, t, blocks, s, query);
+    case 1: return pool_l<T, K, 1, KA>(a, t, blocks, s, query);
+    case 2: return pool_l<T, K, 2, KA>(a, t, blocks, s, query);
+    case 3: return pool_l<T, K, 3, KA>(a, t, blocks, s, query);
+    default: return pool_l<T, K, 4, KA>(a, t, blocks, s, query);
   }
 }
 

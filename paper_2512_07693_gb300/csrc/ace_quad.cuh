@@ -411,22 +411,9 @@ __global__ void __launch_bounds__(kQuadThreads, 1) k_ace_quad(Args<float> a, Ace
 template <typename K, int LMAX>
 int quad_l(const Args<float>* a, const AceDev<float>& t, int blocks, cudaStream_t s, bool query) {
   const size_t bytes = ace_quad_smem<LMAX>(t.nA, t.qrows);
-  if (query) {
-    int dev = 0, optin = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (bytes + (size_t)1024 > (size_t)optin) return 0;
-  }
-  if (cudaFuncSetAttribute(k_ace_quad<K, LMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
-    return 0;
-  if (!query) {
-    launch_pdl(k_ace_quad<K, LMAX>, blocks, kQuadThreads, bytes, s, *a, t);
-    return 0;
-  }
-  int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_ace_quad<K, LMAX>, kQuadThreads, bytes) != cudaSuccess)
-    return 0;
-  return occ;
+  if (query) return resident_blocks(k_ace_quad<K, LMAX>, kQuadThreads, bytes);
+  launch_pdl(k_ace_quad<K, LMAX>, blocks, kQuadThreads, bytes, s, *a, t);
+  return 0;
 }
 
 template <typename K>

@@ -440,19 +440,9 @@ template <typename T, typename K, int LMAX, int GROUP>
 int stream_l(const Args<T>* a, const AceDev<T>& t, int blocks, cudaStream_t s, bool query) {
   const size_t bytes = stream_smem<T, LMAX, GROUP>(t);
   auto kernel = k_ace_stream<T, K, LMAX, GROUP>;
-  if (!query) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    launch_pdl(kernel, blocks, kAceThreads, bytes, s, *a, t);
-    return 0;
-  }
-  int dev = 0, optin = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (bytes + (size_t)1024 > (size_t)optin) return 0;
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return 0;
-  int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, kAceThreads, bytes) != cudaSuccess) return 0;
-  return occ;
+  if (query) return resident_blocks(kernel, kAceThreads, bytes);
+  launch_pdl(kernel, blocks, kAceThreads, bytes, s, *a, t);
+  return 0;
 }
 
 // launch, or occupancy query (resident blocks per SM, 0 if it does not fit), of the kernel

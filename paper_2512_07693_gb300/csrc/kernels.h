@@ -250,6 +250,25 @@ inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
   cudaLaunchKernelEx(&cfg, kernel, static_cast<Act&&>(args)...);
 }
 
+// Resident blocks per SM of a kernel with so many bytes of dynamic shared memory (0: they
+// do not fit), after its limit has been raised to the device's.  The limit belongs to the
+// function, not to the context: with one value for all, contexts of other sizes, in other
+// threads too, launch it without setting it again (each setting it to its own need, one
+// could lower it between another's call and its launch).
+template <typename... KArgs>
+inline int resident_blocks(void (*kernel)(KArgs...), int threads, size_t bytes) {
+  int dev = 0, optin = 0, occ = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  cudaFuncAttributes fa = {};
+  if (bytes + (size_t)1024 > (size_t)optin || cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return 0;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes) !=
+          cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, bytes) != cudaSuccess)
+    return 0;
+  return occ;
+}
+
 template <typename T> Args<T> make_args(apip_ctx* c, const double* pos, const int* id, int n,
                                         double* force, double* e_atom);
 
