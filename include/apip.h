@@ -328,21 +328,26 @@ apip_status apip_check_bounds_selftest(apip_ctx* ctx, void* stream);
  * (host call, no device work).  Body order <= 3 uses the streamed evaluation
  * (couplings C_{(p1 p2) L M} = sum G A_{p1} A_{p2} formed in registers and
  * contracted with their nu = 3 partners), body order 4 the coupling pool (all C
- * of an atom stored, every basis function a dot product of two pool segments; in
- * float32 with ace_group 0 these products as quadratic forms shared by 8 atoms, for
- * which the pool's counts are given).
+ * of an atom stored, every basis function a dot product of two pool segments) or, for
+ * large bases in float32 with ace_group 0, these products as quadratic forms shared by
+ * 8 atoms (where few compacted atoms take the pool all the same, the numbers are those
+ * of the quadratic forms).
  * out (host, APIP_ACE_INFO_COUNT entries):
- *   [0] values per atom in shared memory: 1 + n_max (l_max+1)^2 (+ pool couplings)
- *   [1] couplings (streamed) or coupling components (pool)
+ *   [0] values per atom in shared memory: 1 + n_max (l_max+1)^2 (+ pool couplings);
+ *       quadratic: X and dE/dX of the largest degree, A and dE/dA
+ *   [1] couplings (streamed) or coupling components (pool, quadratic)
  *   [2] Gaunt products per atom (one multiply and one multiply-add each)
- *   [3] basis records (nu = 1, 2 records and nu = 3 partners, or pool records)
- *   [4] sum over the records of their segment length
- *   [5] pool: sum over the pool values of the length of their reverse row
- *   [6] pool: C -> A back-propagation entries
- *   [7] compacted atoms per ACE thread block (streamed with ace_group 0: of a large
- *       system; the kernel takes 2, 4, 8 or 32 by their number)
+ *   [3] basis records (nu = 1, 2 records and nu = 3 partners, or pool records);
+ *       quadratic: tiles of 4 rows
+ *   [4] sum over the records of their segment length; quadratic: multiply-adds per atom
+ *       of phi_2
+ *   [5] pool: sum over the pool values of the length of their reverse row; quadratic:
+ *       multiply-adds per atom of dE/dX (and phi_1)
+ *   [6] pool, quadratic: C -> A back-propagation entries
+ *   [7] compacted atoms per ACE thread block (streamed with ace_group 0: the most, which
+ *       a large system takes; the kernel takes 2, 4, 8 or 32 by their number)
  *   [8] ACE thread blocks per launch
- *   [9] evaluation: 0 = pool, 1 = streamed
+ *   [9] evaluation: 0 = pool, 1 = streamed, 2 = quadratic
  *   [10] floating-point operations per compacted atom of the table work (forward
  *        and adjoint; a multiply-add counts 2); the per-neighbour work is not
  *        included

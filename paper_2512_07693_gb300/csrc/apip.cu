@@ -829,22 +829,42 @@ apip_status apip_create(const apip_params* p, int64_t n_atoms_max, apip_ctx** ou
     ctx->ace_nf = (int)tab.fkey.size();
     ctx->ace_npc = (int)tab.poff.size() - 1;
     int64_t* info = ctx->ace_info;
-    info[0] = tab.npool;
     info[1] = tab.nC;
     for (int c = 0; c < tab.nC; ++c) info[2] += tab.comp[2 * c + 1] & 255u;
-    info[3] = (int64_t)tab.fkey.size();
-    for (uint32_t l : tab.flen) info[4] += l;
-    for (int q = 1; q < tab.npool; ++q) info[5] += tab.qrow[4 * q + 1] - tab.qrow[4 * q];
-    info[6] = (int64_t)tab.bkey.size();
-    // couplings 3 per Gaunt product, basis records 2 per element + 4 each, reverse
-    // rows 4 per element, C -> A entries 3 each
-    info[10] = 3 * info[2] + 2 * info[4] + 4 * info[3] + 4 * info[5] + 3 * info[6];
+    if (quad) {
+      // the products of the tiles: (row, column, M) entries of S (two channels) and K2,
+      // padding included; per atom X_L and dE/dX_L of the largest degree, A and dE/dA
+      info[0] = 2 * hq.rows + 2 * nA;
+      int64_t s_el = 0, k_el = 0, rows = 0;
+      for (int L = 0; L < kQuadLs; ++L)
+        for (int q = 0; q < hq.hdr[4 * L + 3]; ++q) {
+          const int* tl = hq.tile.data() + 8 * (hq.hdr[4 * L + 2] + q);
+          s_el += (int64_t)(2 * L + 1) * kQuadTile * tl[2];
+          k_el += (int64_t)(2 * L + 1) * kQuadTile * tl[6];
+          rows += (int64_t)(2 * L + 1) * tl[7];
+        }
+      info[3] = (int64_t)hq.tile.size() / 8;
+      info[4] = k_el;
+      info[5] = 2 * s_el;
+      info[6] = 2 * info[2];   // (each product to both of its factors)
+      // a multiply-add per entry, 2 per row and phi, 2 for dE/dX; the couplings 3 per
+      // Gaunt product, formed twice, and 3 per product back onto A
+      info[10] = 2 * (info[4] + info[5]) + 6 * rows + 6 * info[2] + 3 * info[6];
+    } else {
+      info[0] = tab.npool;
+      info[3] = (int64_t)tab.fkey.size();
+      for (uint32_t l : tab.flen) info[4] += l;
+      for (int q = 1; q < tab.npool; ++q) info[5] += tab.qrow[4 * q + 1] - tab.qrow[4 * q];
+      info[6] = (int64_t)tab.bkey.size();
+      // couplings 3 per Gaunt product, basis records 2 per element + 4 each, reverse
+      // rows 4 per element, C -> A entries 3 each
+      info[10] = 3 * info[2] + 2 * info[4] + 4 * info[3] + 4 * info[5] + 3 * info[6];
+    }
   }
   // (streamed without a group asked for: the group of a large system)
-  ctx->ace_info[7] = quad ? kQuadAtoms : ctx->ace_group != 0 ? ctx->ace_group
-                     : p->lam_mode == APIP_LAM_PAPER || p->lam_mode == APIP_LAM_LEARNED ? 8 : 32;
-  ctx->ace_info[8] = quad ? ctx->quad_blocks : ctx->ace_blocks;
-  ctx->ace_info[9] = streamed ? 1 : 0;
+  ctx->ace_info[7] = quad ? kQuadAtoms : ctx->ace_group != 0 ? ctx->ace_group : ctx->ace_top;
+  ctx->ace_info[8] = quad ? ctx->quad_blocks : ctx->ace_grid[1] > 0 ? ctx->ace_grid[3] : ctx->ace_blocks;
+  ctx->ace_info[9] = ctx->ace_kind;
   APIP_ALLOC(ctx->ace_tab, host.size());
 #undef APIP_ALLOC
   if (p->precision == APIP_FP64 && p->lam_mode != APIP_LAM_LEARNED) {   // (the learned pass 1 keeps none)
