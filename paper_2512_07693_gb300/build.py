@@ -17,8 +17,9 @@ OUT_DIR_CHECKED = os.path.join(PKG, "_build_checked")
 LIB_CHECKED = os.path.join(PKG, "libapip_checked.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["apip.cu", "kernels_atoms.cu", "kernels_ace_f32.cu", "kernels_ace_f64.cu", "kernels_ace4_f32.cu", "kernels_ace3_f32.cu",
-           "kernels_ace3_f64.cu", "ace_tables.cpp", "apip_static.cu", "kernels_mlp.cu", "peak_probe.cu", "kernels_train_tc.cu"]
+SOURCES = ["apip.cu", "kernels_atoms.cu", "kernels_ace_f32.cu", "kernels_ace_f64.cu", "kernels_ace4_f32.cu",
+           "kernels_ace3_f32.cu", "kernels_ace3_f64.cu", "kernels_ace3l4_f32.cu", "kernels_ace3l4_f64.cu",
+           "ace_tables.cpp", "apip_static.cu", "kernels_mlp.cu", "peak_probe.cu", "kernels_train_tc.cu"]
 HEADERS = ["apip_internal.h", "device_common.cuh", "kernels.h", "ace_device.cuh", "ace_pool.cuh", "ace_quad.cuh", "ace_stream.cuh",
            "gaunt_layout.h", "pair2.cuh", "tc_common.cuh"]
 

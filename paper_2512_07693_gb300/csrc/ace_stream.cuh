@@ -466,7 +466,7 @@ int stream_dispatch(const Args<T>* a, const AceDev<T>& t, int group, int blocks,
     case 1: return stream_g<T, K, 1>(a, t, group, blocks, s, query);
     case 2: return stream_g<T, K, 2>(a, t, group, blocks, s, query);
     case 3: return stream_g<T, K, 3>(a, t, group, blocks, s, query);
-    default: return stream_g<T, K, 4>(a, t, group, blocks, s, query);
+    default: return ace_stream_l4<T>(a, t, group, blocks, s, query);
   }
 }
 

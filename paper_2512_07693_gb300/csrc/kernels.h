@@ -334,5 +334,9 @@ int ace_quad_occupancy(const AceDev<float>& ace);
 template <typename T> cudaError_t ace_stream_set_consts(const double* norms, int count, const double* gaunt);
 template <typename T> void launch_ace_stream(const Args<T>& a, const AceDev<T>& ace, cudaStream_t s);
 template <typename T> int ace_stream_occupancy(const AceDev<T>& ace);
+// its l_max = 4 kernels (kernels_ace3l4_f32.cu, kernels_ace3l4_f64.cu): launch or occupancy query
+template <typename T> cudaError_t ace_stream_l4_set_consts(const double* norms, int count, const double* gaunt);
+template <typename T> int ace_stream_l4(const Args<T>* a, const AceDev<T>& ace, int group, int blocks, cudaStream_t s,
+                                        bool query);
 
 }  // namespace apip

@@ -1,4 +1,4 @@
-// float instantiation of the body-order <= 3 ACE kernel (ace_stream.cuh).
+// float instantiation of the body-order <= 3 ACE kernel (ace_stream.cuh), l_max <= 3.
 #include <vector>
 
 #include "apip_internal.h"
@@ -23,7 +23,8 @@ template <> cudaError_t ace_stream_set_consts<float>(const double* norms, int co
   std::vector<float> f(norms, norms + count), gv(gaunt, gaunt + kGauntTotal);
   const cudaError_t e = cudaMemcpyToSymbol(c_norm, f.data(), sizeof(float) * count);
   if (e != cudaSuccess) return e;
-  return cudaMemcpyToSymbol(c_gaunt, gv.data(), sizeof(float) * kGauntTotal);
+  const cudaError_t e2 = cudaMemcpyToSymbol(c_gaunt, gv.data(), sizeof(float) * kGauntTotal);
+  return e2 != cudaSuccess ? e2 : ace_stream_l4_set_consts<float>(norms, count, gaunt);
 }
 
 template <> void launch_ace_stream<float>(const Args<float>& a, const AceDev<float>& t, cudaStream_t s) {

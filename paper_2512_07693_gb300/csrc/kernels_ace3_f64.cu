@@ -1,4 +1,4 @@
-// double instantiation of the body-order <= 3 ACE kernel (ace_stream.cuh).
+// double instantiation of the body-order <= 3 ACE kernel (ace_stream.cuh), l_max <= 3.
 #include <vector>
 
 #include "apip_internal.h"
@@ -23,7 +23,8 @@ template <> cudaError_t ace_stream_set_consts<double>(const double* norms, int c
   std::vector<double> f(norms, norms + count), gv(gaunt, gaunt + kGauntTotal);
   const cudaError_t e = cudaMemcpyToSymbol(c_norm, f.data(), sizeof(double) * count);
   if (e != cudaSuccess) return e;
-  return cudaMemcpyToSymbol(c_gaunt, gv.data(), sizeof(double) * kGauntTotal);
+  const cudaError_t e2 = cudaMemcpyToSymbol(c_gaunt, gv.data(), sizeof(double) * kGauntTotal);
+  return e2 != cudaSuccess ? e2 : ace_stream_l4_set_consts<double>(norms, count, gaunt);
 }
 
 template <> void launch_ace_stream<double>(const Args<double>& a, const AceDev<double>& t, cudaStream_t s) {
