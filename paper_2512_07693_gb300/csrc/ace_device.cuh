@@ -1,5 +1,5 @@
-// Device code shared by the two ACE kernels (ace_pool.cuh for body order 4,
-// ace_stream.cuh for body order <= 3): real spherical harmonics, the radial
+// Device code shared by the three ACE kernels (ace_pool.cuh and ace_quad.cuh for body
+// order 4, ace_stream.cuh for body order <= 3): real spherical harmonics, the radial
 // basis, table loads, and the per-block steps that do not depend on how the
 // product basis is evaluated:
 //  1. A_nlm = a_scale sum_j R_n(r_ij) Y_lm(rhat_ij) for a group of NAT compacted

@@ -1,4 +1,4 @@
-// ACE evaluation for body order 4 in float32 (the quadratic kernel).  A block takes
+// ACE evaluation for large bases of body order 4 in float32 (the quadratic kernel).  A block takes
 // 8 compacted atoms at a time.  For one degree L, the couplings
 //   C_{(p q) L M} = sum G(l_p m1, l_q m2, L M) A_{p m1} A_{q m2},
 // the segments A_{n L} and, for L = 0, the constant 1 are the rows of X_L (one value
@@ -21,7 +21,7 @@
 // crack's faces).  Compensating within a row (every 16 or 32 columns) cost half and a
 // third more time for nothing beyond that.
 //
-// What bounds it: the loads of the matrix products.  They take 3.45 M multiply-adds per
+// What bounds it: the loads of the matrix products.  They take 3.47 M multiply-adds per
 // atom for n_max 8, l_max 4 (2.95 M on entries that are not zero).  The record-wise pool
 // kernel (ace_pool.cuh) reads its 16-byte records, 5 MB forward and 20 MB back, once
 // per group of 1 to 4 atoms through L2; here 2.1 MB of values serve 8 atoms.  A thread's

@@ -72,15 +72,15 @@ struct SwP { double r_w, r_w_lo, d_lo, d_hi, d0, inv_w, inv_d; };  // 1/(r_w - r
 template <typename T> struct alignas(sizeof(T) == 4 ? 16 : 8) Rec { uint32_t key, len; T k1, k2; };
 template <typename T> struct alignas(sizeof(T) == 4 ? 8 : 16) Ent { T v; uint32_t key; };
 
-// ACE tables on the device.  Two evaluations:
-//  pool (body order 4, built by build_coupled): per atom the pool
+// ACE tables on the device.  Three evaluations:
+//  pool (body order 4 but large bases in float32, built by build_coupled): per atom the pool
 //    X = [1 | A (nA) | C (nC)] holds the atomic density and its Gaunt couplings,
 //    every basis function is the dot product of two pool segments;
 //  streamed (body order <= 3, built by build_streamed): the couplings are formed
 //    one at a time in registers and contracted with their nu = 3 partners; nu = 1, 2
 //    functions are dot products of A segments.
-//  quadratic (body order 4 in float32, built by build_quad): the couplings of one
-//    degree L and the A segments of that degree are the rows of a matrix X_L, and
+//  quadratic (large bases of body order 4 in float32, built by build_quad): the
+//    couplings of one degree L and the A segments of that degree are the rows of a matrix X_L, and
 //    every function of that degree is an entry of a symmetric matrix S_L shared by
 //    all atoms: phi_c = sum_L 1/2 X_L . (S_L^c X_L).
 constexpr int kAcePool = 0, kAceStreamed = 1, kAceQuad = 2;
@@ -94,7 +94,7 @@ constexpr int kQuadMap = (kLmaxCap + 1) * (kLmaxCap + 1) * kNmaxCap * kNmaxCap; 
 
 template <typename T>
 struct AceDev {
-  int kind;                     // kAcePool or kAceStreamed
+  int kind;                     // kAcePool, kAceStreamed or kAceQuad
   int n_max, l_max, nA, nC, npool;   // nA = n_max (l_max+1)^2, npool = 1 + nA + nC
   T rc, rc_lo, eps, sqrt_eps, a_scale;
   T two_over_rc, inv_width;     // 2 / rc and 1 / (rc - rc_lo) of the radial basis

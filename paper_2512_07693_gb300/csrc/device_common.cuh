@@ -5,6 +5,7 @@
 
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <cstdint>
 #include <cstring>
 
@@ -85,12 +86,22 @@ template <> __device__ __forceinline__ double fexp<double>(double x) { return ex
 // function takes some 25 on this GPU's slow float64 pipe.  Outside |x| < 690 (and for
 // a NaN) the library's.
 constexpr int kExpTab = 256;
+// The table: 2^(j / 256) rounded, and what that leaves to 60 binary places.
+inline void exp_table_fill(double2* h) {
+  for (int j = 0; j < kExpTab; ++j) {
+    const long double v = exp2l((long double)j / kExpTab);
+    const double hi = (double)v;
+    h[j] = make_double2(hi, (double)(rintl((v - (long double)hi) * 0x1p60L) * 0x1p-60L));
+  }
+}
 static __device__ __noinline__ double exp_far(double x) { return exp(x); }
 __device__ __forceinline__ double exp_tab(const double2* tab, double x) {
   if ((unsigned)(__double2hiint(x) & 0x7fffffff) >= 0x40859000u) return exp_far(x);
   constexpr double kLn2 = 0.69314718055994530942, kMagic = 6755399441055744.0;   // 1.5 2^52
   constexpr double kStep = kLn2 / kExpTab;
-  constexpr double kHi = (double)(long long)(kStep * 281474976710656.0) / 281474976710656.0;   // 39 bits: k kHi is exact
+  // the first 40 bits of ln2 / 256; x - k kHi is a multiple of x's last place or of 2^-48 and
+  // less than 2^-9, so the multiply-add gives it exactly (k kHi alone would round)
+  constexpr double kHi = (double)(long long)(kStep * 281474976710656.0) / 281474976710656.0;
   constexpr double kLo = 2.8792978770186714e-15;   // ln2 / 256 - kHi
   const double t = fma(x, kExpTab / kLn2, kMagic);
   const int n = __double2loint(t);
@@ -119,13 +130,6 @@ template <> struct Acc<double> {
   double s = 0.0;
   __device__ __forceinline__ void add(double v) { s += v; }
   __device__ __forceinline__ double value() const { return s; }
-};
-
-// Plain running sum (the same interface as Acc).
-template <typename T> struct Plain {
-  T s = T(0);
-  __device__ __forceinline__ void add(T v) { s += v; }
-  __device__ __forceinline__ T value() const { return s; }
 };
 
 // x < y for non-negative doubles by their bit patterns (they order as integers):

@@ -1462,15 +1462,10 @@ template <typename T> void launch_pass1(const Args<T>& a, cudaStream_t s) {
   else launch_pdl(k_pass1<T, 1>, nblocks(a.n, pt), pt, 0, s, a);
 }
 
-// The table of exp_tab on the current device: 2^(j / 256) rounded, and what that
-// leaves to 60 binary places.
+// The table of exp_tab on the current device.
 cudaError_t exp_table_set() {
   std::vector<double2> h(kExpTab);
-  for (int j = 0; j < kExpTab; ++j) {
-    const long double v = exp2l((long double)j / kExpTab);
-    const double hi = (double)v;
-    h[j] = make_double2(hi, (double)(rintl((v - (long double)hi) * 0x1p60L) * 0x1p-60L));
-  }
+  exp_table_fill(h.data());
   return cudaMemcpyToSymbol(g_exp_tab, h.data(), sizeof(double2) * kExpTab);
 }
 
