@@ -21,17 +21,19 @@
 // crack's faces).  Compensating within a row (every 16 or 32 columns) cost half and a
 // third more time for nothing beyond that.
 //
-// What bounds it: the loads of the matrix products.  They take 3.47 M multiply-adds per
-// atom for n_max 8, l_max 4 (2.95 M on entries that are not zero).  The record-wise pool
-// kernel (ace_pool.cuh) reads its 16-byte records, 5 MB forward and 20 MB back, once
-// per group of 1 to 4 atoms through L2; here 2.1 MB of values serve 8 atoms.  A thread's
-// tile is 4 rows (both channels) by the 8 atoms of one M: 32 packed multiply-adds for
-// two uniform 16-byte loads of values and two of X from shared memory (8 rows by 4
-// atoms: four and one, and every load of 16 bytes a lane takes four cycles or more of
-// the load pipe however few addresses it has).  8 atoms are what X_L and dE/dX_L of
-// the largest degree leave room for (2 x 89 KB); step 2 before step 3 instead of both
-// channels' dE/dX_L kept apart costs a fifth more multiply-adds and saves twice that
-// space.  Prefetching the values into L1 one to six steps ahead changed nothing.
+// What bounds it: the matrix products, 3.47 M multiply-adds per atom for n_max 8, l_max 4
+// (2.95 M on entries that are not zero), one barrier after another: a degree's items do
+// not fill the rounds of 384 threads evenly, and the warps wait at the barriers for 4.1 of
+// some 8 cycles per issued instruction (FMA pipe 31 %, L1 42 %, L2 4 % busy, a crack of
+// 126 k atoms).  The record-wise pool kernel (ace_pool.cuh) reads its 16-byte records,
+// 5 MB forward and 20 MB back, once per group of 1 to 4 atoms through L2; here 2.1 MB of
+// values serve 8 atoms.  A thread's tile is 4 rows (both channels) by the 8 atoms of one
+// M: 32 packed multiply-adds for two uniform 16-byte loads of values and two of X from
+// shared memory (8 rows by 4 atoms: four and one, which took 15 % longer).  8 atoms are
+// what X_L and dE/dX_L of the largest degree leave room for (2 x 89 KB); step 2 before
+// step 3 instead of both channels' dE/dX_L kept apart costs a fifth more multiply-adds
+// and saves twice that space.  Prefetching the values into L1 one to six steps ahead
+// changed nothing.
 #pragma once
 
 #include "ace_device.cuh"

@@ -208,7 +208,7 @@ __global__ void k_cell_sort(Args<T> a) {
 //    1357 -> 1050 us).
 //  - FP64 path: the scan tests float positions relative to the cell (the bound is
 //    2e-5 wider than r_list, far above their rounding); only the kept entries see
-//    float64 arithmetic (249 k atoms: 3870 -> 2150 us per build).
+//    float64 arithmetic (249 k atoms: 3870 -> 650 us per build).
 //  - FP32 path, one thread per atom: k_nbfill_one below.
 constexpr unsigned kClassShift = 30;   // n_atoms_max <= 2^30: two bits are free above an index
 template <typename T>
@@ -623,7 +623,7 @@ __global__ void k_set_csp(const int32_t* src, int* dst, int n, int nnb) {
 // of an atom takes the entries s0 + g, s0 + g + LANES, ...
 //
 // FP32 path: two entries at a time, packed (pair2.cuh), the records of the next two
-// in flight meanwhile (pass 2 at 249 k atoms: 70 -> 58 us).  f(s of the first, record, record, count of valid entries: 1 or 2).
+// in flight meanwhile (pass 2 at 249 k atoms: 70 -> 56 us).  f(s of the first, record, record, count of valid entries: 1 or 2).
 template <int LANES, typename L, typename F>
 __device__ __forceinline__ void walk_pairs(const int* nb, int nmax, int s0, int s1, int g, int* status, int n, L&& load,
                                            F&& f) {
