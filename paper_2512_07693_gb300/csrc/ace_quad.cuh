@@ -256,26 +256,42 @@ __device__ __forceinline__ void quad_onto_a(const AceDev<float>& t, int L, const
 }
 
 // Sums of f (pairs of atoms) over the block per atom, with what the compensated sums
-// still have to give back, in red[0 .. 7] after the barrier.
+// still have to give back, in red[0 .. 7] after the barrier.  Each exchange within a warp
+// halves the atoms that a lane keeps (9 float-float additions; 40 with all 8 on every
+// lane).
 __device__ __forceinline__ void quad_sum(const Acc2 (&f)[kQuadAtoms / 2], float* red) {
   constexpr int NW = kQuadThreads / 32;
+  static_assert(kQuadAtoms == 8 && NW % 4 == 0, "three halvings; a quarter of the warps per lane");
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  auto other = [](FF v, int o) { return FF{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)}; };
+  FF v[kQuadAtoms];
 #pragma unroll
   for (int j = 0; j < kQuadAtoms; ++j) {
     const float2 s = f2_get(f[j / 2].s), n = f2_get(f[j / 2].n);
-    FF v = (j & 1) ? FF{s.y, n.y} : FF{s.x, n.x};
+    v[j] = (j & 1) ? FF{s.y, n.y} : FF{s.x, n.x};
+  }
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1)
-      v = ff_add(v, FF{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)});
-    if (lane == 0) {
-      red[warp * kQuadAtoms + j] = v.hi;
-      red[(NW + warp) * kQuadAtoms + j] = v.lo;
+  for (int o = 16, keep = 4; keep > 0; o >>= 1, keep >>= 1)
+#pragma unroll
+    for (int j = 0; j < keep; ++j) {
+      const bool up = (lane & o) != 0;
+      const FF mine = up ? v[j + keep] : v[j];
+      v[j] = ff_add(mine, other(up ? v[j] : v[j + keep], o));
     }
+#pragma unroll
+  for (int o = 2; o > 0; o >>= 1) v[0] = ff_add(v[0], other(v[0], o));
+  if ((lane & 3) == 0) {   // lane 4 a: atom a
+    red[warp * kQuadAtoms + lane / 4] = v[0].hi;
+    red[(NW + warp) * kQuadAtoms + lane / 4] = v[0].lo;
   }
   __syncthreads();
   FF t{0.f, 0.f};
-  if (tid < kQuadAtoms)
-    for (int w = 0; w < NW; ++w) t = ff_add(t, FF{red[w * kQuadAtoms + tid], red[(NW + w) * kQuadAtoms + tid]});
+  if (warp == 0) {
+    for (int w = lane / kQuadAtoms; w < NW; w += 32 / kQuadAtoms)
+      t = ff_add(t, FF{red[w * kQuadAtoms + lane % kQuadAtoms], red[(NW + w) * kQuadAtoms + lane % kQuadAtoms]});
+#pragma unroll
+    for (int o = kQuadAtoms; o < 32; o <<= 1) t = ff_add(t, other(t, o));
+  }
   __syncthreads();
   if (tid < kQuadAtoms) red[tid] = t.hi + t.lo;
   __syncthreads();
